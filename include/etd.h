@@ -58,21 +58,20 @@ typedef enum {
 typedef enum { ETD_ETDRK1 = 1, ETD_ETDRK2 = 2 } etd_scheme;   /* EIFE1 eq. (2.13), EIFE2 eq. (2.14) */
 typedef enum { ETD_F64 = 0, ETD_F32 = 1 } etd_dtype;            /* arithmetic and storage type of u */
 /* Transform implementation of the DST-I along each axis.
- * ETD_ROUTE_FFT: FP32 uses the odd extension (a length-2N complex FFT per pair of pencils; rounding
- *   grows like log N); FP64 uses the half-length recurrence below.
- * ETD_ROUTE_FFT_HALF: a length-N complex FFT per pair of pencils followed by a prefix sum (half the
- *   work; rounding grows like sqrt(N/2) eps).
- * ETD_ROUTE_AUTO: per axis, FP32 takes ETD_ROUTE_FFT for N >= 512 and ETD_ROUTE_FFT_HALF below;
- *   FP64 always takes the recurrence.
+ * ETD_ROUTE_AUTO, ETD_ROUTE_FFT, ETD_ROUTE_FFT_HALF: Dirichlet axes of length 32 and more run the odd
+ *   extension (a length-2N complex FFT per pair of pencils; rounding grows like log N) folded to the half
+ *   its symmetry leaves, FP32 and FP64. Shorter axes: FP32 on ETD_ROUTE_FFT the plain odd extension,
+ *   otherwise the half-length recurrence (a length-N complex FFT per pair of pencils followed by a
+ *   prefix sum; rounding grows like sqrt(N/2) eps).
  * ETD_ROUTE_FFT_SPLIT (FP32; otherwise as ETD_ROUTE_AUTO): Dirichlet axes of N = 1024 (strided ones when
  *   N[0] is a multiple of 4) run a split-radix DST-I: the odd outputs are a DST-III of length N/2, the
  *   even ones split once more into a DST-III of length N/4 and a DST-I of length N/4, each computed by a
  *   complex FFT that fits in one warp (512, 256 and 512 points per pair of pencils against 2048 for the
  *   odd extension; rounding grows like log N, and is smaller than the odd extension's in practice).
  *   Exact arithmetic equal to the other FFT routes; batches take it as ETD_ROUTE_AUTO.
- * FP32 2D plans on the FFT routes take the phi-function weights of the stage combinations from per-mode
- * tables of FP64 values rounded once to FP32 (12 bytes per unknown for EIFE2, 4 for EIFE1, up to 64 MiB;
- * larger and 3D plans evaluate them per mode in FP32).
+ * 2D plans on the FFT routes take the phi-function weights of the stage combinations from per-mode
+ * tables of FP64 values rounded once to the plan's type (FP32: 12 bytes per unknown for EIFE2, 4 for
+ * EIFE1; up to 64 MiB; larger and 3D plans and batches evaluate them per mode in the plan's type).
  * ETD_ROUTE_GEMM_TF32 and ETD_ROUTE_GEMM_BF16X3 (FP32 plans only; every N[a] a multiple of 32):
  *   the DST-I along an axis is the dense product with the N x N sine matrix S_a of Section 4 (periodic
  *   plans: the N x N orthonormal Hartley matrix),

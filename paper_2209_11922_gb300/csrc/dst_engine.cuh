@@ -53,7 +53,41 @@ template <class T> __device__ __forceinline__ Cx<T> operator*(T s, Cx<T> a) { re
 template <class T> __device__ __forceinline__ Cx<T> cmul(Cx<T> a, Cx<T> b) {
   return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};
 }
-template <class T> __device__ __forceinline__ Cx<T> mul_i(Cx<T> a) { return {-a.y, a.x}; }
+template <class T> __device__ __forceinline__ Cx<T> mul2(Cx<T> a, Cx<T> b) { return {a.x * b.x, a.y * b.y}; }  // component-wise
+template <class T> __device__ __forceinline__ Cx<T> fma2(Cx<T> a, Cx<T> b, Cx<T> c) { return {a.x * b.x + c.x, a.y * b.y + c.y}; }
+template <class T> __device__ __forceinline__ Cx<T> add_i(Cx<T> a, Cx<T> b) { return {a.x - b.y, a.y + b.x}; }  // a + i b
+template <class T> __device__ __forceinline__ Cx<T> sub_i(Cx<T> a, Cx<T> b) { return {a.x + b.y, a.y - b.x}; }  // a - i b
+
+// FP32: both components in one packed instruction (add / mul / fma .f32x2, two IEEE single operations each): these
+// kernels are bound by instruction issue, and the component-wise operations are most of a butterfly.
+union F32x2 {
+  Cx<float> c;
+  unsigned long long u;
+};
+__device__ __forceinline__ Cx<float> operator+(Cx<float> a, Cx<float> b) {
+  F32x2 x, y, r;
+  x.c = a;
+  y.c = b;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.u) : "l"(x.u), "l"(y.u));
+  return r.c;
+}
+__device__ __forceinline__ Cx<float> mul2(Cx<float> a, Cx<float> b) {
+  F32x2 x, y, r;
+  x.c = a;
+  y.c = b;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.u) : "l"(x.u), "l"(y.u));
+  return r.c;
+}
+__device__ __forceinline__ Cx<float> fma2(Cx<float> a, Cx<float> b, Cx<float> c) {
+  F32x2 x, y, z, r;
+  x.c = a;
+  y.c = b;
+  z.c = c;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.u) : "l"(x.u), "l"(y.u), "l"(z.u));
+  return r.c;
+}
+__device__ __forceinline__ Cx<float> operator-(Cx<float> a, Cx<float> b) { return fma2(b, Cx<float>{-1.f, -1.f}, a); }
+__device__ __forceinline__ Cx<float> operator*(float s, Cx<float> a) { return mul2(Cx<float>{s, s}, a); }
 
 // cos(2 pi m / 96) for 0 <= m <= 24 (quarter wave), then by symmetry for any m >= 0.
 __host__ __device__ constexpr double qcos96(int m) {
@@ -109,53 +143,61 @@ template <class T, int M> __device__ __forceinline__ Cx<T> twmul96(Cx<T> v) {
   else if constexpr (m == 72) return {v.y, -v.x};
   else {
     constexpr T c = (T)cos96(m), s = (T)sin96(m);
-    return {c * v.x - s * v.y, c * v.y + s * v.x};
+    const Cx<T> w = c * v;
+    return {w.x - s * v.y, w.y + s * v.x};
   }
 }
 
-// In-register DFT of length R with kernel exp(+2 pi i r k / R), natural order in and out.
-template <class T, int R> struct Dft {
+// In-register DFT of length R with kernel exp(+2 pi i r k / R), natural order in and out. NI: the second half of
+// the input (index >= R/2) is given negated; NO: the second half of the output is returned negated. Both cost
+// nothing (the signs go into the first or last butterflies); R must then split so that the halves fall to the
+// inner (NI) or outer (NO) factor's halves.
+template <class T, int R, bool NI = false, bool NO = false> struct Dft {
   static_assert(96 % R == 0, "radix must divide 96");
-  static constexpr int F = (R % 4 == 0) ? 4 : (R % 2 == 0 ? 2 : 3);
+  static constexpr int F = (NI && R % 3 == 0) ? 3 : (R % 4 == 0) ? 4 : (R % 2 == 0 ? 2 : 3);
   static constexpr int Q = R / F;
+  static_assert(!NI || Q % 2 == 0, "negated input half");
+  static_assert(!NO || F % 2 == 0, "negated output half");
   static __device__ __forceinline__ void run(Cx<T>* x);
 };
-template <class T> struct Dft<T, 1> { static __device__ __forceinline__ void run(Cx<T>*) {} };
-template <class T> struct Dft<T, 2> {
+template <class T, bool NI, bool NO> struct Dft<T, 1, NI, NO> { static __device__ __forceinline__ void run(Cx<T>*) {} };
+template <class T, bool NI, bool NO> struct Dft<T, 2, NI, NO> {
   static __device__ __forceinline__ void run(Cx<T>* x) {
     const Cx<T> a = x[0], b = x[1];
-    x[0] = a + b;
-    x[1] = a - b;
+    x[0] = NI ? a - b : a + b;
+    x[1] = NI ? (NO ? Cx<T>{-a.x - b.x, -a.y - b.y} : a + b) : (NO ? b - a : a - b);
   }
 };
-template <class T> struct Dft<T, 3> {
+template <class T, bool NI, bool NO> struct Dft<T, 3, NI, NO> {
+  static_assert(!NI && !NO, "odd length has no halves");
   static __device__ __forceinline__ void run(Cx<T>* x) {
     const Cx<T> s = x[1] + x[2], d = x[1] - x[2];
     const Cx<T> t = x[0] - T(0.5) * s;
-    const Cx<T> u = mul_i(T(0.86602540378443864676) * d);
+    const Cx<T> u = T(0.86602540378443864676) * d;
     x[0] = x[0] + s;
-    x[1] = t + u;
-    x[2] = t - u;
+    x[1] = add_i(t, u);
+    x[2] = sub_i(t, u);
   }
 };
-template <class T> struct Dft<T, 4> {
+template <class T, bool NI, bool NO> struct Dft<T, 4, NI, NO> {
   static __device__ __forceinline__ void run(Cx<T>* x) {
-    const Cx<T> a0 = x[0] + x[2], a1 = x[0] - x[2], b0 = x[1] + x[3], b1 = mul_i(x[1] - x[3]);
+    const Cx<T> s02 = x[0] + x[2], d02 = x[0] - x[2], s13 = x[1] + x[3], d13 = x[1] - x[3];
+    const Cx<T> a0 = NI ? d02 : s02, a1 = NI ? s02 : d02, b0 = NI ? d13 : s13, b1 = NI ? s13 : d13;
     x[0] = a0 + b0;
-    x[2] = a0 - b0;
-    x[1] = a1 + b1;
-    x[3] = a1 - b1;
+    x[1] = add_i(a1, b1);
+    x[2] = NO ? b0 - a0 : a0 - b0;
+    x[3] = NO ? Cx<T>{-a1.x - b1.y, b1.x - a1.y} : sub_i(a1, b1);
   }
 };
-template <class T, int R>
-__device__ __forceinline__ void Dft<T, R>::run(Cx<T>* x) {
+template <class T, int R, bool NI, bool NO>
+__device__ __forceinline__ void Dft<T, R, NI, NO>::run(Cx<T>* x) {
   Cx<T> y[F][Q];
 #pragma unroll
   for (int s = 0; s < F; ++s)
 #pragma unroll
     for (int q = 0; q < Q; ++q) y[s][q] = x[F * q + s];
 #pragma unroll
-  for (int s = 0; s < F; ++s) Dft<T, Q>::run(y[s]);
+  for (int s = 0; s < F; ++s) Dft<T, Q, NI, false>::run(y[s]);
   static_for<0, Q>([&](auto kc) {
     constexpr int k = decltype(kc)::value;
     Cx<T> a[F];
@@ -163,7 +205,7 @@ __device__ __forceinline__ void Dft<T, R>::run(Cx<T>* x) {
       constexpr int s = decltype(sc)::value;
       a[s] = twmul96<T, (96 / R) * s * k>(y[s][k]);
     });
-    Dft<T, F>::run(a);
+    Dft<T, F, false, NO>::run(a);
 #pragma unroll
     for (int t = 0; t < F; ++t) x[k + Q * t] = a[t];
   });
@@ -175,8 +217,9 @@ __device__ __forceinline__ void Dft<T, R>::run(Cx<T>* x) {
 template <int... Rs> struct Radices {};
 template <class T, int N, bool ODD> struct FftPlan;
 // Transform variant of a kernel (template argument VAR): the two DST-I forms and the Hartley form.
-// The Hartley variant runs the recurrence variant's length-N FFT plan.
-enum Variant : int { V_REC = 0, V_ODD = 1, V_HART = 2 };
+// The Hartley variant runs the recurrence variant's length-N FFT plan; V_FOLD names the folded odd extension
+// of fold_dst.cuh, which has kernels of its own.
+enum Variant : int { V_REC = 0, V_ODD = 1, V_HART = 2, V_FOLD = 3 };
 #define ETD_PLAN(TYPE, NN, ODD_, TPP_, ...)                \
   template <> struct FftPlan<TYPE, NN, ODD_> {             \
     static constexpr bool ODD = ODD_;                      \

@@ -19,6 +19,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -31,6 +32,7 @@
 
 #include "../../include/etd.h"
 #include "boundary.cuh"
+#include "fold_pass.cuh"
 #include "gemm_pass.cuh"
 #include "monitor.cuh"
 #include "pass_kernel.cuh"
@@ -97,6 +99,16 @@ int env_int(const char* name, int dflt) {
   return (v && *v) ? atoi(v) : dflt;
 }
 
+// Transform variant of an axis of length n: periodic axes the Hartley kernels; Dirichlet axes the folded odd
+// extension, which is exact in the same sense as both DST-I forms below and does less work than either, and
+// the lengths it has no plan for (below 32, 24 included) the odd extension or the recurrence: FP32 as the route
+// says (AUTO: the recurrence), FP64 the recurrence.
+int dst_variant(const etd_options& o, int64_t n) {
+  if (o.bc == ETD_BC_PERIODIC) return V_HART;
+  if (fold_has((int)n)) return V_FOLD;
+  return o.dtype == ETD_F32 && o.route == ETD_ROUTE_FFT ? V_ODD : V_REC;
+}
+
 bool supported_length(int64_t n) {
   if (n < 4 || n > 2048) return false;
   int64_t m = n;
@@ -134,6 +146,8 @@ struct etd_plan_s {
   const void* zeta[3] = {};
   const void* ex[3] = {};
   const void* ec[3] = {};
+  const void* em[3] = {};
+  const void* cm[3] = {};
   double sc[3] = {};
   std::vector<Launch> step;   // one time step
   cudaStream_t cap_stream = nullptr;
@@ -178,6 +192,8 @@ void fill_common(const etd_plan_s* pl, PassArgs<T>& a) {
     a.zeta[d] = static_cast<const T*>(pl->zeta[d]);
     a.ex[d] = static_cast<const T*>(pl->ex[d]);
     a.ec[d] = static_cast<const T*>(pl->ec[d]);
+    a.em[d] = static_cast<const T*>(pl->em[d]);
+    a.cm[d] = static_cast<const T*>(pl->cm[d]);
   }
   a.tau = (T)pl->tau;
   a.c2 = (T)pl->opt.c2;
@@ -243,6 +259,91 @@ etd_status make_split_launch(etd_plan_s* pl, int op, int axis, const void* in0, 
   return ETD_OK;
 }
 
+// Dense user field <-> pitched field (PACK / UNPACK): four rows per round and block, their loads in flight together.
+template <class T>
+__global__ void __launch_bounds__(256) pack_kernel(const PassArgs<T> A) {
+  griddep_wait();
+  constexpr int U = 4;
+  const int cut = A.user_slot;   // 1: Dirichlet (index 0 is the boundary), 0: periodic
+  const int rows = A.ny * A.nz;
+  for (int r0 = blockIdx.x; r0 < rows; r0 += U * gridDim.x) {
+    long long d[U];   // dense start of the row, -1: boundary row or past the end
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int r = r0 + u * gridDim.x, z = r / A.ny, y = r - z * A.ny;
+      const bool in = r < rows && y >= cut && (A.ndim == 2 || z >= cut);
+      d[u] = in ? ((long long)(A.ndim == 3 ? z - cut : 0) * (A.ny - cut) + (y - cut)) * (A.nx - cut) - cut : -2;
+    }
+    for (int x = threadIdx.x; x < A.nx; x += blockDim.x) {
+      T v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const bool in = d[u] > -2 && x >= cut;
+        v[u] = T(0);
+        if (in) v[u] = A.op == OP_PACK ? A.in0[d[u] + x] : A.in0[(size_t)(r0 + u * gridDim.x) * A.nx + x];
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (A.op == OP_PACK) {
+          if (r0 + u * (int)gridDim.x < rows) A.out0[(size_t)(r0 + u * gridDim.x) * A.nx + x] = v[u];
+        } else if (d[u] > -2 && x >= cut) {
+          A.out0[d[u] + x] = v[u];
+        }
+      }
+    }
+  }
+}
+
+// One pass on the folded odd extension (fold_pass.cuh).
+template <class T>
+etd_status make_fold_launch(etd_plan_s* pl, const KernelInfo* k, PassArgs<T>& a, int kind, double fields_rw, Launch& L) {
+  const int op = a.op;
+  int P = 16;
+  while (P * k->tpp > k->max_threads) P /= 2;
+  long long grid = 0;
+  int optin = 0;
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, pl->device);
+  const bool tab = fold_is_stage(op) && a.coef;
+  if (a.axis == 0) {
+    a.npairs = pl->ny * pl->nz / 2;
+    // Where step B's units are 8 threads (L >= 64) four pairs: unit 0 of step B, which runs other code, is then a warp of its
+    // own instead of a part of one.
+    const int pmin = k->radix[1] >= 64 ? 4 : 1;
+    while (P > pmin && (a.npairs + P - 1) / P < 2 * pl->num_sms) P /= 2;
+    grid = (a.npairs + P - 1) / P;
+  } else {
+    // A tile's row segment (2P values) is at least one 32-byte sector
+    const int other = (a.axis == 1) ? pl->nz : pl->ny;
+    const int pmin = k->radix[1] >= 64 ? 4 : 16 / (int)sizeof(T);
+    while (P > pmin && (pl->nx / (2 * P)) * (long long)other < 2 * pl->num_sms) P /= 2;
+    while (P > 1 && (pl->nx % (2 * P) != 0 || fold_smem_bytes(*k, op, P, pair_stride(*k, P), tab, false) > (size_t)optin)) P /= 2;
+    if (pl->nx % (2 * P) != 0) return fail(ETD_ERR_UNSUPPORTED, "x extent %d not even", pl->nx);
+    a.tiles_x = pl->nx / (2 * P);
+    grid = (long long)a.tiles_x * other;
+  }
+  a.P = P;
+  a.lp = pair_stride(*k, P);
+  if (tab) {
+    const size_t staged = fold_smem_bytes(*k, op, P, a.lp, true, true);
+    a.coef_smem = staged <= (size_t)optin ? 1 : 0;
+  }
+  L.fn = tab ? k->fn_tab[op] : (op == OP_TRANSFORM && a.axis == 0 ? k->fn_x : k->fn_op[op]);
+  if (!L.fn) return fail(ETD_ERR_UNSUPPORTED, "no kernel for pass %d of axis length %d", op, k->N);
+  L.grid = dim3((unsigned)grid);
+  L.block = dim3((unsigned)(P * k->tpp));
+  L.smem = fold_smem_bytes(*k, op, P, a.lp, tab, a.coef_smem != 0);
+  L.kind = kind;
+  memcpy(L.args, &a, sizeof(a));
+  L.args_size = sizeof(a);
+  L.alg_bytes = fields_rw * (double)pl->unknowns * sizeof(T);
+  if (L.smem > (size_t)optin) return fail(ETD_ERR_UNSUPPORTED, "tile needs %zu B of shared memory (max %d)", L.smem, optin);
+  if (L.smem > 48 * 1024) {   // the device maximum: one kernel serves launches with different tile sizes
+    cudaError_t e = cudaFuncSetAttribute(L.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+    if (e != cudaSuccess) return fail(ETD_ERR_CUDA, "cudaFuncSetAttribute(%d B): %s", optin, cudaGetErrorString(e));
+  }
+  return ETD_OK;
+}
+
 template <class T>
 etd_status make_launch(etd_plan_s* pl, int op, int axis, const void* in0, const void* in1, void* out0,
                        void* out1, int kind, double fields_rw, Launch& L) {
@@ -257,6 +358,22 @@ etd_status make_launch(etd_plan_s* pl, int op, int axis, const void* in0, const 
   if (!k) return fail(ETD_ERR_UNSUPPORTED, "no kernel for axis length %d", N);
   PassArgs<T> a;
   fill_common<T>(pl, a);
+  if (op == OP_PACK || op == OP_UNPACK) {
+    a.op = op;
+    a.in0 = static_cast<const T*>(in0);
+    a.out0 = static_cast<T*>(out0);
+    a.user_slot = pl->periodic ? 0 : 1;
+    const long long blocks = ((long long)pl->ny * pl->nz + 3) / 4;   // four rows each
+    L.fn = reinterpret_cast<const void*>(&pack_kernel<T>);
+    L.grid = dim3((unsigned)(blocks < 16LL * pl->num_sms ? blocks : 16LL * pl->num_sms));
+    L.block = dim3(256);
+    L.smem = 0;
+    L.kind = kind;
+    memcpy(L.args, &a, sizeof(a));
+    L.args_size = sizeof(a);
+    L.alg_bytes = fields_rw * (double)pl->unknowns * sizeof(T);
+    return ETD_OK;
+  }
   a.op = op;
   a.axis = axis;
   a.in0 = static_cast<const T*>(in0);
@@ -272,6 +389,7 @@ etd_status make_launch(etd_plan_s* pl, int op, int axis, const void* in0, const 
     else if (op == OP_S2 || op == OP_S2S) a.coef = cf + pl->coef_s2;
     else if (op == OP_RK1 || op == OP_RK1S) a.coef = cf + pl->coef_rk1;
   }
+  if (k->odd == V_FOLD) return make_fold_launch<T>(pl, k, a, kind, fields_rw, L);
   const bool two = (op == OP_RK1 || op == OP_S1 || op == OP_S2 || op == OP_RK1S || op == OP_S1S || op == OP_S2S);
   const int maxp = 512 / k->tpp > 0 ? 512 / k->tpp : 1;
   int P = 1;
@@ -829,19 +947,52 @@ etd_status entry_exit_any(etd_plan_s* pl, bool entry, void* u, std::vector<Launc
   return pl->elem == 4 ? entry_exit<float>(pl, entry, u, out) : entry_exit<double>(pl, entry, u, out);
 }
 
+// Tables of a folded axis (fold_dst.cuh), FP64 values rounded once to T: step A's [R/2][L/2] entries, and for
+// L >= 64 the twiddles exp(2 pi i t i / L) as [L/8][8] and the inner transform's step A entries (R = 16, L/8).
+template <class T>
+void append_fold_twiddles(const KernelInfo* k, std::vector<T>& h) {
+  const double sc = 0.5 * sqrt(2.0 / (double)k->N);
+  auto put = [&](double x, double y) {
+    h.push_back((T)x);
+    h.push_back((T)y);
+  };
+  auto step_a = [&](int R, int Ls) {
+    for (int kk = 0; kk < R / 2; ++kk)
+      for (int jj = 0; jj < Ls / 2; ++jj) {
+        if (kk == 0 && jj == 0) put(0.0, sc);
+        else if (kk == 0) put(sc * sin(M_PI * jj / Ls), 0.5 * sc);
+        else if (jj == 0) put(0.5 * sc / tan(M_PI * kk / R), 0.5 * sc / sin(M_PI * kk / R));
+        else put(sc * sin(2.0 * M_PI * (double)(jj * kk) / ((double)R * Ls)),
+                 -sc * cos(2.0 * M_PI * (double)(jj * kk) / ((double)R * Ls)));
+      }
+  };
+  const int R = k->radix[0], Ls = k->radix[1];
+  step_a(R, Ls);
+  if (Ls >= 64) {
+    for (int i = 0; i < Ls / 8; ++i)
+      for (int t = 0; t < 8; ++t) put(cos(2.0 * M_PI * t * i / Ls), sin(2.0 * M_PI * t * i / Ls));
+    step_a(16, Ls / 8);
+  }
+}
+
 // FP64 on the host, rounded once to T, appended to h for one axis of length n: the per-pass twiddle
 // tables (pass with NS > 1 and radix R holds exp(2 pi i k r / (NS R)) at [(r-1)*NS + k], k < NS,
 // r = 1..R-1, the layout the Stockham passes read), sin(pi j / n), and per mode i the values
-// zeta = tau D mu_i, exp(-zeta), exp(-c2 zeta) with mu_i = (6/h^2)(1 - cos)/(2 + cos) of theta = i pi / n
+// zeta = tau D mu_i, exp(-zeta), exp(-c2 zeta), 1 - exp(-zeta), 1 - exp(-c2 zeta) with mu_i = (6/h^2)(1 - cos)/(2 + cos) of theta = i pi / n
 // (periodic axes: theta = 2 pi i / n, mode 0 included with zeta = 0).
-// offs receives the five table starts (element offsets into h).
+// offs receives the seven table starts (element offsets into h).
 template <class T>
 void append_axis_tables(const KernelInfo* k, int n, double hh, double tauD, double c2, std::vector<T>& h,
-                        size_t offs[5], bool periodic = false) {
+                        size_t offs[7], bool periodic = false) {
+  while (h.size() % 4) h.push_back(T(0));   // complex entries aligned for 8- and 16-byte copies
   offs[0] = h.size();
   int NS = 1;
   size_t t = 0;
-  for (int i = 0; i < 4 && k->radix[i]; ++i) {
+  if (k->odd == V_FOLD) {
+    append_fold_twiddles<T>(k, h);
+    t = 1;
+  }
+  for (int i = 0; k->odd != V_FOLD && i < 4 && k->radix[i]; ++i) {
     const int R = k->radix[i];
     if (NS > 1) {
       for (int r = 1; r < R; ++r)
@@ -860,10 +1011,9 @@ void append_axis_tables(const KernelInfo* k, int n, double hh, double tauD, doub
   }
   offs[1] = h.size();
   for (int j = 0; j < n; ++j) h.push_back((T)sin(M_PI * (double)j / (double)n));
-  offs[2] = h.size();
-  offs[3] = offs[2] + n;
-  offs[4] = offs[2] + 2 * (size_t)n;
-  h.resize(h.size() + 3 * (size_t)n);
+  while (h.size() % 2) h.push_back(T(0));   // per-mode values read in adjacent pairs
+  for (int t = 2; t < 7; ++t) offs[t] = h.size() + (size_t)(t - 2) * n;
+  h.resize(h.size() + 5 * (size_t)n);
   for (int i = 0; i < n; ++i) {
     double zeta = 0.0;
     if (i > 0) {
@@ -875,6 +1025,8 @@ void append_axis_tables(const KernelInfo* k, int n, double hh, double tauD, doub
     h[offs[2] + i] = (T)zeta;
     h[offs[3] + i] = (T)exp(-zeta);
     h[offs[4] + i] = (T)exp(-c2 * zeta);
+    h[offs[5] + i] = (T)-expm1(-zeta);
+    h[offs[6] + i] = (T)-expm1(-c2 * zeta);
   }
 }
 
@@ -903,7 +1055,7 @@ size_t append_split_tables(std::vector<T>& h) {
 // phi_1(z), phi_2(z) in FP64 for z <= 0 (Section 2.2): the Taylor series sum_m z^m/(m+k)! for |z| < 1/2
 // (24 terms, truncation below 1e-20), the closed forms (e^z - 1)/z and (e^z - 1 - z)/z^2 through expm1
 // above, where their cancellation costs at most a few ulps.
-void phi12_fp64(double z, double& p1, double& p2) {
+__device__ void phi12_fp64(double z, double& p1, double& p2) {
   if (fabs(z) < 0.5) {
     double s1 = 0, s2 = 0, t = 1, f1 = 1, f2 = 0.5;
     for (int m = 0; m < 24; ++m) {
@@ -922,59 +1074,66 @@ void phi12_fp64(double z, double& p1, double& p2) {
   }
 }
 
-// Per-mode phi-function weights of a 2D FP32 plan (FFT routes, both the default and the split-radix
-// kernels read them), computed in FP64 from zeta = tau D (mu_x + mu_y) with the closed-form 1D rates (those of append_axis_tables) and
-// rounded once to FP32; layouts as documented for PassArgs::coef (the exponentials e^{-z}, e^{-c2 z} are
-// products of the per-axis tables).
+// Per-mode phi-function weights of a 2D plan (the default and the split-radix kernels read them), computed in FP64 from
+// zeta = tau D (mu_x + mu_y) with the closed-form 1D rates (those of append_axis_tables) and rounded once to T;
+// layouts as documented for PassArgs::coef (the exponentials e^{-z}, e^{-c2 z} are products of the per-axis tables).
+// On the device: 24 series terms or two expm1 per mode cost the host 0.1 s at 1024^2.
+template <class T>
+__global__ void __launch_bounds__(256) coef_kernel(const double* __restrict__ zx, const double* __restrict__ zy, int nx,
+                                                   long long modes, double tau, double c2, int scheme, T* __restrict__ s1,
+                                                   T* __restrict__ s2) {
+  for (long long m = blockIdx.x * (long long)blockDim.x + threadIdx.x; m < modes; m += (long long)gridDim.x * blockDim.x) {
+    const double z = zx[m % nx] + zy[m / nx];
+    double p1, p2;
+    phi12_fp64(-z, p1, p2);
+    if (scheme == 2) {
+      double p1c, p2c;
+      phi12_fp64(-c2 * z, p1c, p2c);
+      s1[2 * m + 0] = (T)(c2 * tau * p1c);
+      s1[2 * m + 1] = (T)(tau * (p1 - p2 / c2));
+      s2[m] = (T)(tau * p2 / c2);
+    } else {
+      s1[m] = (T)(tau * p1);
+    }
+  }
+}
+
 template <class T>
 etd_status upload_coef_tables(etd_plan_s* pl) {
   const int nx = pl->nx, ny = pl->ny;
   const size_t modes = (size_t)nx * ny;
-  const double tauD = pl->tau * pl->D, c2 = pl->opt.c2, tau = pl->tau;
-  std::vector<double> mx(nx), my(ny);
+  const double tauD = pl->tau * pl->D;
+  std::vector<double> hz((size_t)nx + ny);
   auto mu = [](int i, int n, double hh) {
     if (i == 0) return 0.0;
     const double th = M_PI * (double)i / (double)n, s = sin(0.5 * th);
     return 12.0 / (hh * hh) * s * s / (2.0 + cos(th));   // (6/h^2)(1 - cos)/(2 + cos)
   };
-  for (int i = 0; i < nx; ++i) mx[i] = mu(i, nx, pl->h[0]);
-  for (int j = 0; j < ny; ++j) my[j] = mu(j, ny, pl->h[1]);
-  std::vector<T> h;
-  if (pl->scheme == 2) {
-    pl->coef_s1 = 0;
-    pl->coef_s2 = 2 * modes;
-    h.resize(3 * modes);
-    for (int j = 0; j < ny; ++j)
-      for (int i = 0; i < nx; ++i) {
-        const size_t m = (size_t)j * nx + i;
-        const double z = tauD * (mx[i] + my[j]);
-        double p1, p2, p1c, p2c;
-        phi12_fp64(-z, p1, p2);
-        phi12_fp64(-c2 * z, p1c, p2c);
-        h[2 * m + 0] = (T)(c2 * tau * p1c);
-        h[2 * m + 1] = (T)(tau * (p1 - p2 / c2));
-        h[2 * modes + m] = (T)(tau * p2 / c2);
-      }
-  } else {
-    pl->coef_rk1 = 0;
-    h.resize(modes);
-    for (int j = 0; j < ny; ++j)
-      for (int i = 0; i < nx; ++i) {
-        const size_t m = (size_t)j * nx + i;
-        double p1, p2;
-        phi12_fp64(-tauD * (mx[i] + my[j]), p1, p2);
-        h[m] = (T)(tau * p1);
-      }
+  for (int i = 0; i < nx; ++i) hz[i] = tauD * mu(i, nx, pl->h[0]);
+  for (int j = 0; j < ny; ++j) hz[nx + j] = tauD * mu(j, ny, pl->h[1]);
+  pl->coef_s1 = pl->coef_rk1 = 0;
+  pl->coef_s2 = 2 * modes;
+  ETD_CUDA(cudaMalloc(&pl->coef, (pl->scheme == 2 ? 3 : 1) * modes * sizeof(T)));
+  double* dz = nullptr;
+  ETD_CUDA(cudaMalloc(&dz, hz.size() * sizeof(double)));
+  cudaError_t e = cudaMemcpy(dz, hz.data(), hz.size() * sizeof(double), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) {
+    T* cf = static_cast<T*>(pl->coef);
+    const size_t blocks = std::min<size_t>((modes + 255) / 256, 8 * (size_t)pl->num_sms);
+    coef_kernel<T><<<(unsigned)blocks, 256>>>(dz, dz + nx, nx, (long long)modes, pl->tau, pl->opt.c2, pl->scheme, cf,
+                                              cf + 2 * modes);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
   }
-  ETD_CUDA(cudaMalloc(&pl->coef, h.size() * sizeof(T)));
-  ETD_CUDA(cudaMemcpy(pl->coef, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice));
+  cudaFree(dz);
+  if (e != cudaSuccess) return fail(ETD_ERR_CUDA, "phi-weight tables: %s", cudaGetErrorString(e));
   return ETD_OK;
 }
 
 template <class T>
 etd_status upload_tables(etd_plan_s* pl) {
   std::vector<T> h;
-  size_t offs[3][5], soff[3] = {0, 0, 0};
+  size_t offs[3][7], soff[3] = {0, 0, 0};
   for (int a = 0; a < pl->ndim; ++a) {
     const KernelInfo* k = find_pass_kernel((int)sizeof(T), (int)pl->N[a], pl->odd[a]);
     if (!k) return fail(ETD_ERR_UNSUPPORTED, "no kernel for axis length %lld", (long long)pl->N[a]);
@@ -991,6 +1150,8 @@ etd_status upload_tables(etd_plan_s* pl) {
     pl->zeta[a] = base + offs[a][2];
     pl->ex[a] = base + offs[a][3];
     pl->ec[a] = base + offs[a][4];
+    pl->em[a] = base + offs[a][5];
+    pl->cm[a] = base + offs[a][6];
     pl->stw[a] = pl->split[a] ? base + soff[a] : nullptr;
   }
   for (int a = pl->ndim; a < 3; ++a) {   // unused third axis in 2D: point at axis 0 (never read)
@@ -999,6 +1160,8 @@ etd_status upload_tables(etd_plan_s* pl) {
     pl->zeta[a] = pl->zeta[0];
     pl->ex[a] = pl->ex[0];
     pl->ec[a] = pl->ec[0];
+    pl->em[a] = pl->em[0];
+    pl->cm[a] = pl->cm[0];
   }
   return ETD_OK;
 }
@@ -1126,7 +1289,7 @@ struct etd_batch_s {
 namespace {
 
 struct BatchTables {
-  size_t off[2][5];
+  size_t off[2][7];
   double sc[2];
 };
 
@@ -1146,6 +1309,8 @@ int batch_args(const etd_batch_s* b, const std::vector<BatchTables>& tabs, int i
     a.zeta[d] = base + tabs[i].off[dd][2];
     a.ex[d] = base + tabs[i].off[dd][3];
     a.ec[d] = base + tabs[i].off[dd][4];
+    a.em[d] = base + tabs[i].off[dd][5];
+    a.cm[d] = base + tabs[i].off[dd][6];
   }
   a.tw = base + tabs[i].off[axis][0];
   a.sn = base + tabs[i].off[axis][1];
@@ -1175,6 +1340,11 @@ int batch_args(const etd_batch_s* b, const std::vector<BatchTables>& tabs, int i
   return a.tiles_x;
 }
 
+// Shared memory of a batched launch.
+size_t batch_smem(const KernelInfo& k, int op, int P, int nbuf) {
+  return k.odd == V_FOLD ? fold_smem_bytes(k, op, P, pair_stride(k, P), false, false) : pass_smem_bytes(k, P, nbuf);
+}
+
 template <class T>
 etd_status batch_group_upload(etd_batch_s* b, const std::vector<BatchTables>& tabs, BatchGroup& g, int f_in0,
                               int f_in1, int f_out0, int f_out1, char*& aux_cursor) {
@@ -1186,7 +1356,7 @@ etd_status batch_group_upload(etd_batch_s* b, const std::vector<BatchTables>& ta
     for (int t = 0; t < tiles; ++t) map.push_back(make_int2((int)li, t));
   }
   g.nctas = (int)map.size();
-  g.smem = pass_smem_bytes(*k, g.P, g.nbuf);
+  g.smem = batch_smem(*k, g.op, g.P, g.nbuf);
   const size_t dbytes = descs.size() * sizeof(PassArgs<T>), mbytes = map.size() * sizeof(int2);
   g.d_descs = aux_cursor;
   aux_cursor += (dbytes + 255) & ~(size_t)255;
@@ -1254,8 +1424,9 @@ etd_status batch_build_op(etd_batch_s* b, const std::vector<BatchTables>& tabs, 
     // (strided passes) dividing every problem's x extent
     std::vector<int> cands;
     const size_t budget = (size_t)b->optin / (size_t)k->min_blocks - 2048;
-    for (int P = 1; P * k->tpp <= 512; P *= 2) {
-      if (pass_smem_bytes(*k, P, o.nbuf) > budget) break;
+    const int max_threads = k->odd == V_FOLD ? k->max_threads : 512;
+    for (int P = 1; P * k->tpp <= max_threads; P *= 2) {
+      if (batch_smem(*k, o.op, P, o.nbuf) > (k->odd == V_FOLD ? (size_t)b->optin : budget)) break;
       bool ok = true;
       if (o.axis != 0)
         for (int i : g.inst) ok = ok && (b->nx[i] % (2 * P) == 0);
@@ -1634,19 +1805,14 @@ etd_status etd_plan_create(etd_plan* out, int ndim, const int64_t* N, const doub
   pl->opt = o;
   pl->elem = (o.dtype == ETD_F32) ? 4 : 8;
   for (int a = 0; a < ndim; ++a) {
-    // FP32: the odd extension keeps rounding at log N; AUTO uses it from N = 512 up and the
-    // half-length recurrence (sqrt(N/2) eps <= 11 eps) below, where it is twice as fast.
-    // Periodic axes: the Hartley variant (a plain length-N FFT, rounding like log N) on every route.
-    if (pl->periodic) pl->odd[a] = V_HART;
-    else if (o.dtype != ETD_F32 || o.route == ETD_ROUTE_FFT_HALF) pl->odd[a] = V_REC;
-    else if (o.route == ETD_ROUTE_FFT) pl->odd[a] = V_ODD;
-    else pl->odd[a] = N[a] >= 512 ? V_ODD : V_REC;
+    pl->odd[a] = dst_variant(o, N[a]);
   }
   // ETD_ROUTE_FFT_SPLIT: FP32 Dirichlet axes of length 1024 take the split-radix kernels (the strided
   // passes need an x extent that is a multiple of 4); every other axis the AUTO choice.
   for (int a = 0; a < ndim; ++a)
     pl->split[a] = (o.dtype == ETD_F32 && !pl->periodic && o.route == ETD_ROUTE_FFT_SPLIT && N[a] == SPLIT_N &&
                     (a == 0 || N[0] % 4 == 0)) ? 1 : 0;
+  if (pl->split[ndim - 1]) pl->odd[ndim - 1] = V_ODD;   // its stage passes (no V~) under a source or boundary data
   pl->nx = (int)N[0];
   pl->ny = (int)N[1];
   pl->nz = ndim == 3 ? (int)N[2] : 1;
@@ -1677,7 +1843,7 @@ etd_status etd_plan_create(etd_plan* out, int ndim, const int64_t* N, const doub
   const size_t coef_bytes = pl->nfield * (pl->scheme == 2 ? 3 : 1) * (size_t)pl->elem;
   if (ndim == 2 && !pl->periodic && !gemm && coef_bytes <= ((size_t)64 << 20)) {
     if (pl->elem == 4) st = upload_coef_tables<float>(pl);
-    else if (pl->odd[1] == V_REC && N[1] == 1024) st = upload_coef_tables<double>(pl);
+    else if (pl->odd[1] == V_FOLD) st = upload_coef_tables<double>(pl);
     if (st != ETD_OK) return bail(st);
   }
   if (gemm) {
@@ -2052,12 +2218,8 @@ etd_status etd_batch_create(etd_batch* out, int count, const int64_t* N, const d
     b->hx.push_back(h[2 * i]);
     b->hy.push_back(h[2 * i + 1]);
     b->Dv.push_back(D[i]);
-    auto odd_of = [&](int64_t n) {
-      if (o.bc == ETD_BC_PERIODIC) return (int)V_HART;
-      return (o.dtype != ETD_F32 || o.route == ETD_ROUTE_FFT_HALF) ? 0 : (o.route == ETD_ROUTE_FFT ? 1 : (n >= 512 ? 1 : 0));
-    };
-    b->oddx.push_back(odd_of(N[2 * i]));
-    b->oddy.push_back(odd_of(N[2 * i + 1]));
+    b->oddx.push_back(dst_variant(o, N[2 * i]));
+    b->oddy.push_back(dst_variant(o, N[2 * i + 1]));
   }
   if (cudaGetDevice(&b->device) != cudaSuccess) {
     delete b;

@@ -74,6 +74,8 @@ template <class T> struct PassArgs {
   const T* zeta[3]; // per paper axis: tau D mu_a
   const T* ex[3];   // exp(-tau D mu_a)
   const T* ec[3];   // exp(-c2 tau D mu_a)
+  const T* em[3];   // 1 - exp(-tau D mu_a)
+  const T* cm[3];   // 1 - exp(-c2 tau D mu_a)
   T sc, tau, c2, flin, fcub, flog;
   // Separable time-dependent source of the reaction (REACT passes; src_gx == NULL: none). The pass
   // stores S_x f(u), so it adds src_amp exp(-src_rate t) (S_x g_x)[k] g_y[y] g_z[z] at node row
@@ -118,15 +120,10 @@ template <class T, int N, int VAR> constexpr bool TABLES_ON() { return sizeof(T)
 // (staged before the dependency wait; the host passes no tables where a launch cannot stage them);
 // longer axes read the tables from global memory.
 template <class T, int N, int VAR> constexpr bool TABLES_STAGED() { return TABLES_ON<T, N, VAR>() && N <= 1536; }
-// Shapes with kernels per operation for the passes of a time step (REACT, TRANSFORM, RK1S, S1S, S2S):
-// the FP32 lengths of the large 2D and 3D workloads and of batches of meshes from 64 to 384, and the FP64
-// length of the 2D workloads (N = 1024).
+// Shapes with kernels per operation for the passes of a time step (REACT, TRANSFORM, RK1S, S1S, S2S): the FP32
+// length of the periodic 3D workload. (Dirichlet axes of 32 and more run the kernels of fold_pass.cuh.)
 template <class T, int N, int VAR> constexpr bool pass_op_kernels() {
-  return (sizeof(T) == 4 &&
-          ((VAR == V_ODD && (N == 1024 || N == 2048)) ||
-           (VAR == V_REC && (N == 64 || N == 96 || N == 128 || N == 192 || N == 256 || N == 384)) ||
-           (VAR == V_HART && N == 128))) ||
-         (sizeof(T) == 8 && VAR == V_REC && N == 1024);
+  return sizeof(T) == 4 && VAR == V_HART && N == 128;
 }
 // FP64: the operation-fixed kernels (the 2D FP64 workloads' axis length) read the tables from global memory.
 template <class T, int N, int VAR> constexpr bool TABLES_ANY() {
@@ -671,6 +668,11 @@ struct KernelInfo {
   int twn;      // twiddle table entries
   int radix[4]; // Stockham radices (0-terminated)
   int min_blocks;  // CTAs per SM the register budget was compiled for
+  // folded-odd-extension kernels (odd == V_FOLD: fn_op and fn_batched_op only)
+  const void* fn_tab[OP_COUNT];  // stage passes reading per-mode weight tables
+  const void* fn_x;              // OP_TRANSFORM along x
+  int max_threads;               // CTA size limit
+  int own_vals;                  // values a thread holds after step B
 };
 
 template <int... Rs> void radix_list(int* out, Radices<Rs...>) {
