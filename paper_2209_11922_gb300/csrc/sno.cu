@@ -14,6 +14,7 @@
 #include "../../include/etd.h"
 #include "../../include/etd_sno.h"
 #include "sno_kernels.cuh"
+#include "sno_layer.cuh"
 #include "sno_mma.cuh"
 
 void etd_internal_set_error(const char* msg);   // etd_api.cu
@@ -78,6 +79,10 @@ struct etd_sno_s {
   // forward contractions on the tensor cores (BF16 operands, FP32 accumulation) when every K and output
   // width fits a tile (n, C <= 256); the backward keeps FP32 (the exact straight-through gradient)
   bool tc = false;
+  int fused_mp = 0;        // inference by the fused layers (sno_layer.cuh): modes per axis padded to 16 or 24, 0: not
+  uint2* Sf = nullptr;     // S_M as bf16 fragments
+  float* Ty = nullptr;     // [Bmax][n y][C][MP]
+  float* Tx = nullptr;     // [Bmax][n x][C][MP]
   int num_sms = 148;
   int* err = nullptr;      // set by a tensor-core kernel whose wait ran out
 };
@@ -265,13 +270,14 @@ etd_status upload_feature(etd_sno_s* m, const double* D, int B, cudaStream_t s) 
 namespace {
 
 void sno_free(etd_sno_s* m) {
-  float* bufs[] = {m->W, m->G, m->Mo, m->Ve, m->S, m->a, m->T, m->gh, m->dgh, m->dh0, m->dh1, m->uhat, m->du, m->part};
+  float* bufs[] = {m->W, m->G, m->Mo, m->Ve, m->S, m->a, m->T, m->Ty, m->Tx, m->gh, m->dgh, m->dh0, m->dh1, m->uhat, m->du, m->part};
   for (float* p : bufs)
     if (p) cudaFree(p);
   for (float* p : m->h) cudaFree(p);
   for (float* p : m->z) cudaFree(p);
   for (float* p : m->hh) cudaFree(p);
   if (m->lpart) cudaFree(m->lpart);
+  if (m->Sf) cudaFree(m->Sf);
   if (m->err) cudaFree(m->err);
   if (m->ahost) cudaFreeHost(m->ahost);
   delete m;
@@ -346,6 +352,58 @@ etd_status sno_forward(etd_sno_s* m, const float* u, int B, float* out, cudaStre
   project_kernel<<<dim3(pblk, B), 256, 0, s>>>(u, m->h[L], m->W + m->oWq, m->W + m->obq, out, C, np);
   SNO_CUDA(cudaGetLastError());
   return ETD_OK;
+}
+
+// Inference by the fused layers: channels-last fields ping-pong between h[0] and h[1].
+template <int C, int MP, bool FIRST, bool LAST>
+etd_status launch_layer(const LayerArgs& g, cudaStream_t s) {
+  const size_t smem = layer_smem<C, MP, FIRST, LAST>();
+  SNO_CUDA(cudaFuncSetAttribute(layer_kernel<C, MP, FIRST, LAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  layer_kernel<C, MP, FIRST, LAST><<<dim3((g.n + LY - 1) / LY, g.B), 256, smem, s>>>(g);
+  SNO_CUDA(cudaGetLastError());
+  return ETD_OK;
+}
+template <int C, int MP>
+etd_status sno_infer(etd_sno_s* m, const float* u, int B, float* out, cudaStream_t s) {
+  const int n = m->n, M = m->M, L = m->L;
+  LayerArgs g{};
+  g.B = B;
+  g.n = n;
+  g.M = M;
+  g.u = u;
+  g.a = m->a;
+  g.Wl = m->W + m->oWl;
+  g.bl = m->W + m->obl;
+  g.S = m->S;
+  g.Sf = m->Sf;
+  g.T = m->Ty;
+  g.Tf = m->Tx;
+  g.Wq = m->W + m->oWq;
+  g.bq = m->W + m->obq;
+  g.out = out;
+  lift_modes_kernel<C, MP><<<dim3(std::min((n + 7) / 8, std::max(1, 4 * m->num_sms / B)), B), 256, 0, s>>>(g);
+  SNO_CUDA(cudaGetLastError());
+  SNO_CUDA(cudaFuncSetAttribute(modes_y_kernel<MP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)modes_y_smem(n, MP)));
+  for (int l = 0; l < L; ++l) {
+    modes_y_kernel<MP><<<dim3((C * MP + 127) / 128, B), 256, modes_y_smem(n, MP), s>>>(m->S, m->Ty, m->hh[0], B, n, M, C);
+    SNO_CUDA(cudaGetLastError());
+    mode_mix_kernel<C><<<M * M, 256, 0, s>>>(m->W + m->oWm + (long long)l * M * M * C * C, m->hh[0], m->gh, B);
+    SNO_CUDA(cudaGetLastError());
+    modes_x_kernel<MP><<<dim3((C * MP + 255) / 256, B, (n + 63) / 64), 256, 0, s>>>(m->S, m->gh, m->Tx, B, n, M, C);
+    SNO_CUDA(cudaGetLastError());
+    g.Wp = m->W + m->oWp + (long long)l * C * C;
+    g.bp = m->W + m->obp + (long long)l * C;
+    g.h = m->h[l & 1];
+    g.hn = m->h[(l + 1) & 1];
+    const bool first = l == 0, last = l == L - 1;
+    SNO_TRY(first ? (last ? launch_layer<C, MP, true, true>(g, s) : launch_layer<C, MP, true, false>(g, s))
+                  : (last ? launch_layer<C, MP, false, true>(g, s) : launch_layer<C, MP, false, false>(g, s)));
+  }
+  return ETD_OK;
+}
+etd_status sno_infer_any(etd_sno_s* m, const float* u, int B, float* out, cudaStream_t s) {
+  if (m->C == 32) return m->fused_mp == 16 ? sno_infer<32, 16>(m, u, B, out, s) : sno_infer<32, 24>(m, u, B, out, s);
+  return m->fused_mp == 16 ? sno_infer<16, 16>(m, u, B, out, s) : sno_infer<16, 24>(m, u, B, out, s);
 }
 
 // sum over fields and pixels of X[b][c][i] * (y ? y[b][i] : 1), weighted per field by w (device,
@@ -492,6 +550,18 @@ etd_status etd_sno_create(etd_sno* out, int N, int C, int M, int L, int max_batc
   if (cudaMemcpy(m->S, hs.data(), hs.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess)
     return bail(sfail(ETD_ERR_CUDA, "upload of the mode matrix"));
   m->tc = m->n <= 256 && C <= 256 && M <= 256;
+  // Fused inference layers: channel counts and mode counts whose fragments fit the registers (C = 16 or 32, M <= 24)
+  // and rows whose bf16 S_M fits beside the tiles; they round the operands that the tensor-core path rounds, so only
+  // where that path runs.
+  if (m->tc && (C == 16 || C == 32) && M <= 24) {
+    m->fused_mp = M <= 16 ? 16 : 24;
+    const long long cnt = (long long)max_batch * m->n * C * m->fused_mp;
+    const std::vector<uint2> f = s_fragments(hs, M, m->fused_mp, m->n);
+    if (cudaMalloc(&m->Sf, f.size() * sizeof(uint2)) != cudaSuccess ||
+        cudaMemcpy(m->Sf, f.data(), f.size() * sizeof(uint2), cudaMemcpyHostToDevice) != cudaSuccess)
+      return bail(sfail(ETD_ERR_OOM, "mode-matrix fragments"));
+    if ((st = sno_alloc(&m->Ty, cnt)) != ETD_OK || (st = sno_alloc(&m->Tx, cnt)) != ETD_OK) return bail(st);
+  }
   int dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&m->num_sms, cudaDevAttrMultiProcessorCount, dev);
@@ -525,6 +595,7 @@ etd_status etd_sno_forward(etd_sno m, const float* u, const double* D, int B, fl
   if (out == u) return sfail(ETD_ERR_INVALID_ARG, "out may not alias u");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   SNO_TRY(upload_feature(m, D, B, s));
+  if (m->fused_mp) return sno_infer_any(m, u, B, out, s);
   return sno_forward(m, u, B, out, s, false);
 }
 
