@@ -25,6 +25,8 @@ LIB = os.path.join(LIBDIR, "libetd_gb300.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 LENGTHS = [4, 8, 16, 32, 64, 128, 256, 512, 1024, 2048, 6, 12, 24, 48, 96, 192, 384, 768, 1536]
 FOLD = [32, 48, 64, 96, 128, 192, 256, 384, 512, 768, 1024, 1536, 2048]   # fold_has() of fold_dst.cuh
+# foldh_has() of fold_dst.cuh
+FOLDH = {"f32": [32, 48, 64, 96, 128, 192, 256, 384, 512], "f64": []}
 TYPES = {"f32": "float", "f64": "double"}
 
 
@@ -52,22 +54,23 @@ def generate() -> list:
     srcs = []
     decls, rows = [], []
     for tk, tn in TYPES.items():
-        # transform variants (enum Variant of dst_engine.cuh): 2 Hartley (periodic axes); Dirichlet axes the
-        # folded odd extension (3), and where it has no plan 1 odd extension (FP32 only; 1024 for the
-        # split-radix route's plans) and 0 half-length recurrence
-        for n in FOLD:
-            name = f"kinfo_{tk}_fold_{n}"
-            path = os.path.join(GEN, f"inst_{tk}_fold_{n}.cu")
-            _write_if_changed(path, (
-                '#include "fold_pass.cuh"\n'
-                "namespace etd {\n"
-                f"KernelInfo {name}() {{ return fold_info<{tn}, {n}>(); }}\n"
-                "}  // namespace etd\n"))
-            srcs.append(path)
-            decls.append(f"KernelInfo {name}();")
-            rows.append(f"    {name}(),")
+        # transform variants (enum Variant of dst_engine.cuh): the two-step kernels (Dirichlet axes 3, periodic axes 4),
+        # and for lengths without a two-step plan 2 Hartley, 1 odd extension (FP32 only; 1024 for the split-radix route's
+        # plans) and 0 half-length recurrence
+        for v, per, lengths in (("fold", "false", FOLD), ("foldh", "true", FOLDH[tk])):
+            for n in lengths:
+                name = f"kinfo_{tk}_{v}_{n}"
+                path = os.path.join(GEN, f"inst_{tk}_{v}_{n}.cu")
+                _write_if_changed(path, (
+                    '#include "fold_pass.cuh"\n'
+                    "namespace etd {\n"
+                    f"KernelInfo {name}() {{ return fold_info<{tn}, {n}, {per}>(); }}\n"
+                    "}  // namespace etd\n"))
+                srcs.append(path)
+                decls.append(f"KernelInfo {name}();")
+                rows.append(f"    {name}(),")
         for v, o in ((("odd", 1), ("rec", 0), ("hart", 2)) if tk == "f32" else (("rec", 0), ("hart", 2))):
-            for n in LENGTHS if v == "hart" else [m for m in LENGTHS if m not in FOLD] + [1024] * (v == "odd"):
+            for n in [m for m in LENGTHS if m not in ([m for m in FOLDH[tk] if m != 512] if v == "hart" else FOLD)] + [1024] * (v == "odd"):
                 name = f"kinfo_{tk}_{v}_{n}"
                 path = os.path.join(GEN, f"inst_{tk}_{v}_{n}.cu")
                 _write_if_changed(path, (

@@ -99,15 +99,18 @@ int env_int(const char* name, int dflt) {
   return (v && *v) ? atoi(v) : dflt;
 }
 
-// Transform variant of an axis of length n: periodic axes the Hartley kernels; Dirichlet axes the folded odd
+// Transform variant of an axis of length n with `pairs` pencil pairs: periodic axes the two-step Hartley kernels where they have a plan, else the
+// general Hartley kernels; Dirichlet axes the folded odd
 // extension, which is exact in the same sense as both DST-I forms below and does less work than either, and
 // the lengths it has no plan for (below 32, 24 included) the odd extension or the recurrence: FP32 as the route
 // says (AUTO: the recurrence), FP64 the recurrence.
-int dst_variant(const etd_options& o, int64_t n) {
-  if (o.bc == ETD_BC_PERIODIC) return V_HART;
+int dst_variant(const etd_options& o, int64_t n, int64_t pairs) {
+  if (o.bc == ETD_BC_PERIODIC) return foldh_has(o.dtype == ETD_F32 ? 4 : 8, (int)n, pairs) ? V_FOLDH : V_HART;
   if (fold_has((int)n)) return V_FOLD;
   return o.dtype == ETD_F32 && o.route == ETD_ROUTE_FFT ? V_ODD : V_REC;
 }
+
+bool two_step(const KernelInfo& k) { return k.odd == V_FOLD || k.odd == V_FOLDH; }
 
 bool supported_length(int64_t n) {
   if (n < 4 || n > 2048) return false;
@@ -389,7 +392,7 @@ etd_status make_launch(etd_plan_s* pl, int op, int axis, const void* in0, const 
     else if (op == OP_S2 || op == OP_S2S) a.coef = cf + pl->coef_s2;
     else if (op == OP_RK1 || op == OP_RK1S) a.coef = cf + pl->coef_rk1;
   }
-  if (k->odd == V_FOLD) return make_fold_launch<T>(pl, k, a, kind, fields_rw, L);
+  if (two_step(*k)) return make_fold_launch<T>(pl, k, a, kind, fields_rw, L);
   const bool two = (op == OP_RK1 || op == OP_S1 || op == OP_S2 || op == OP_RK1S || op == OP_S1S || op == OP_S2S);
   const int maxp = 512 / k->tpp > 0 ? 512 / k->tpp : 1;
   int P = 1;
@@ -967,6 +970,15 @@ void append_fold_twiddles(const KernelInfo* k, std::vector<T>& h) {
       }
   };
   const int R = k->radix[0], Ls = k->radix[1];
+  if (k->odd == V_FOLDH) {   // w_N^{jj k} at [k][jj]; entry (0, 0): 1/(2 sqrt N)
+    for (int kk = 0; kk < R; ++kk)
+      for (int jj = 0; jj < Ls; ++jj) {
+        const double t = 2.0 * M_PI * (double)(jj * kk) / (double)k->N;
+        if (kk == 0 && jj == 0) put(0.0, 0.5 / sqrt((double)k->N));
+        else put(cos(t), sin(t));
+      }
+    return;
+  }
   step_a(R, Ls);
   if (Ls >= 64) {
     for (int i = 0; i < Ls / 8; ++i)
@@ -988,11 +1000,11 @@ void append_axis_tables(const KernelInfo* k, int n, double hh, double tauD, doub
   offs[0] = h.size();
   int NS = 1;
   size_t t = 0;
-  if (k->odd == V_FOLD) {
+  if (two_step(*k)) {
     append_fold_twiddles<T>(k, h);
     t = 1;
   }
-  for (int i = 0; k->odd != V_FOLD && i < 4 && k->radix[i]; ++i) {
+  for (int i = 0; !two_step(*k) && i < 4 && k->radix[i]; ++i) {
     const int R = k->radix[i];
     if (NS > 1) {
       for (int r = 1; r < R; ++r)
@@ -1104,9 +1116,9 @@ etd_status upload_coef_tables(etd_plan_s* pl) {
   const size_t modes = (size_t)nx * ny;
   const double tauD = pl->tau * pl->D;
   std::vector<double> hz((size_t)nx + ny);
-  auto mu = [](int i, int n, double hh) {
+  auto mu = [&](int i, int n, double hh) {
     if (i == 0) return 0.0;
-    const double th = M_PI * (double)i / (double)n, s = sin(0.5 * th);
+    const double th = (pl->periodic ? 2.0 : 1.0) * M_PI * (double)i / (double)n, s = sin(0.5 * th);
     return 12.0 / (hh * hh) * s * s / (2.0 + cos(th));   // (6/h^2)(1 - cos)/(2 + cos)
   };
   for (int i = 0; i < nx; ++i) hz[i] = tauD * mu(i, nx, pl->h[0]);
@@ -1342,7 +1354,7 @@ int batch_args(const etd_batch_s* b, const std::vector<BatchTables>& tabs, int i
 
 // Shared memory of a batched launch.
 size_t batch_smem(const KernelInfo& k, int op, int P, int nbuf) {
-  return k.odd == V_FOLD ? fold_smem_bytes(k, op, P, pair_stride(k, P), false, false) : pass_smem_bytes(k, P, nbuf);
+  return two_step(k) ? fold_smem_bytes(k, op, P, pair_stride(k, P), false, false) : pass_smem_bytes(k, P, nbuf);
 }
 
 template <class T>
@@ -1424,9 +1436,9 @@ etd_status batch_build_op(etd_batch_s* b, const std::vector<BatchTables>& tabs, 
     // (strided passes) dividing every problem's x extent
     std::vector<int> cands;
     const size_t budget = (size_t)b->optin / (size_t)k->min_blocks - 2048;
-    const int max_threads = k->odd == V_FOLD ? k->max_threads : 512;
+    const int max_threads = two_step(*k) ? k->max_threads : 512;
     for (int P = 1; P * k->tpp <= max_threads; P *= 2) {
-      if (batch_smem(*k, o.op, P, o.nbuf) > (k->odd == V_FOLD ? (size_t)b->optin : budget)) break;
+      if (batch_smem(*k, o.op, P, o.nbuf) > (two_step(*k) ? (size_t)b->optin : budget)) break;
       bool ok = true;
       if (o.axis != 0)
         for (int i : g.inst) ok = ok && (b->nx[i] % (2 * P) == 0);
@@ -1805,7 +1817,7 @@ etd_status etd_plan_create(etd_plan* out, int ndim, const int64_t* N, const doub
   pl->opt = o;
   pl->elem = (o.dtype == ETD_F32) ? 4 : 8;
   for (int a = 0; a < ndim; ++a) {
-    pl->odd[a] = dst_variant(o, N[a]);
+    pl->odd[a] = dst_variant(o, N[a], N[0] * N[1] * (ndim == 3 ? N[2] : 1) / N[a] / 2);
   }
   // ETD_ROUTE_FFT_SPLIT: FP32 Dirichlet axes of length 1024 take the split-radix kernels (the strided
   // passes need an x extent that is a multiple of 4); every other axis the AUTO choice.
@@ -1838,12 +1850,10 @@ etd_status etd_plan_create(etd_plan* out, int ndim, const int64_t* N, const doub
   for (int f = 0; f < nf; ++f) pl->F[f] = static_cast<char*>(pl->ws) + f * fbytes;
   etd_status st = (pl->elem == 4) ? upload_tables<float>(pl) : upload_tables<double>(pl);
   if (st != ETD_OK) return bail(st);
-  // per-mode phi-function weights of the y passes of 2D plans on the FFT routes (at most 64 MiB): FP32
-  // plans, and FP64 plans whose y axis runs the FP64 operation-fixed kernels (N = 1024), which read them
+  // per-mode phi-function weights of the y passes of 2D plans on the FFT routes (at most 64 MiB)
   const size_t coef_bytes = pl->nfield * (pl->scheme == 2 ? 3 : 1) * (size_t)pl->elem;
-  if (ndim == 2 && !pl->periodic && !gemm && coef_bytes <= ((size_t)64 << 20)) {
-    if (pl->elem == 4) st = upload_coef_tables<float>(pl);
-    else if (pl->odd[1] == V_FOLD) st = upload_coef_tables<double>(pl);
+  if (ndim == 2 && !gemm && coef_bytes <= ((size_t)64 << 20)) {
+    st = pl->elem == 4 ? upload_coef_tables<float>(pl) : upload_coef_tables<double>(pl);
     if (st != ETD_OK) return bail(st);
   }
   if (gemm) {
@@ -2218,8 +2228,8 @@ etd_status etd_batch_create(etd_batch* out, int count, const int64_t* N, const d
     b->hx.push_back(h[2 * i]);
     b->hy.push_back(h[2 * i + 1]);
     b->Dv.push_back(D[i]);
-    b->oddx.push_back(dst_variant(o, N[2 * i]));
-    b->oddy.push_back(dst_variant(o, N[2 * i + 1]));
+    b->oddx.push_back(dst_variant(o, N[2 * i], 1024));   // the group's pairs of all problems fill the GPU
+    b->oddy.push_back(dst_variant(o, N[2 * i + 1], 1024));
   }
   if (cudaGetDevice(&b->device) != cudaSuccess) {
     delete b;

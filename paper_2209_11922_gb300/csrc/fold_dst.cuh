@@ -341,7 +341,7 @@ template <class T, int N> struct Fold {
       }
     }
   }
-  static __device__ __forceinline__ void b_end(const C* __restrict__ bp, int s, C (&z)[VB]) {
+  static __device__ __forceinline__ void b_end(const C* __restrict__ bp, int s, C (&z)[VB], const C* __restrict__) {
     if constexpr (!BIG) {
       const C* p = bp + s * LS;
 #pragma unroll
@@ -372,7 +372,7 @@ template <class T, int N> struct Fold {
     }
   }
   // Transposes, in the slots that b_end / b_mid read.
-  static __device__ __forceinline__ void bt_begin(C* __restrict__ bp, int s, C (&z)[VB]) {
+  static __device__ __forceinline__ void bt_begin(C* __restrict__ bp, int s, C (&z)[VB], const C* __restrict__) {
     if constexpr (!BIG) {
       fold_bt<T, L>(z, s == 0);
       C* p = bp + s * LS;
@@ -431,6 +431,177 @@ template <class T, int N> struct Fold {
 #pragma unroll
         for (int i = 0; i < VB; ++i) p[i * (8 + 8 / G)] = x[i];
       }
+    }
+  }
+};
+
+// ---------------------------------------------------------------------------------------------
+// Periodic axes: the Hartley transform of dst_engine.cuh in the same two steps (N = R L). A: radix-R butterflies
+// jj = 0..L-1 over z[jj + r L], y_k[jj] = w_N^{jj k} X_k left in the slots it read (k L + jj). B: the DFT of length L of
+// y_k gives Z at R m + k; H needs Z_n and Z_{N-n} together, which units k and R - k hold, so a thread runs both (unit 0
+// with unit R/2, each paired with itself), 2 L values. The transform is symmetric, so its transpose is the same
+// transform: the combination's transpose, then B and A with the conjugate kernel, which is the same kernel between two
+// swaps of the components.
+template <class T, int N> struct FoldHPlan { static constexpr int R = 0, L = 0, TPP = 1, G = 1; };
+#define ETD_FOLDH(NN, R_, L_, G_)                                                  \
+  template <class T> struct FoldHPlan<T, NN> {                                     \
+    static_assert(R_ * L_ == NN, "R L = N");                                       \
+    static constexpr int R = R_, L = L_, TPP = L_, G = G_;                         \
+  };
+ETD_FOLDH(32, 8, 4, 4)
+ETD_FOLDH(48, 12, 4, 4)
+ETD_FOLDH(64, 16, 4, 4)
+ETD_FOLDH(96, 24, 4, 4)
+ETD_FOLDH(128, 16, 8, 8)
+ETD_FOLDH(192, 24, 8, 8)
+ETD_FOLDH(256, 32, 8, 8)
+ETD_FOLDH(384, 24, 16, 16)
+ETD_FOLDH(512, 32, 16, 16)
+#undef ETD_FOLDH
+
+// FP32 only: FP64 passes cost their longest thread (see the plans above), and the general Hartley kernels hold half the
+// values per thread up to 128 (64^2 ETDRK2: 159 us per step against 204); at 128^3, where every thread is busy, the two
+// are equal (1378 and 1404). N = 512 (32 values per thread) needs enough pairs to fill the SMs: 512^2 with 256 pairs
+// takes 28.9 us against 26.5.
+constexpr bool foldh_has(int elem, int n, long long pairs) {
+  return elem == 4 && (n == 32 || n == 48 || n == 64 || n == 96 || n == 128 || n == 192 || n == 256 || n == 384 ||
+                       (n == 512 && pairs >= 1024));
+}
+
+template <class T> __device__ __forceinline__ Cx<T> swp(Cx<T> a) { return {a.y, a.x}; }
+
+template <class T, int N> struct FoldH {
+  using Plan = FoldHPlan<T, N>;
+  using C = Cx<T>;
+  static constexpr int R = Plan::R, L = Plan::L, TPP = Plan::TPP, G = Plan::G;
+  static constexpr int H = R / 2;
+  static constexpr int UA = L;
+  static constexpr bool BIG = false;
+  static constexpr int SLOTS = H, QB = (SLOTS + TPP - 1) / TPP;
+  static constexpr int VB = 2 * L, HV = L, STEP = R;
+  static constexpr int LP = N + N / G;
+  static constexpr int TWN = R * L;   // w_N^{jj k} at [k][jj]; entry (0, 0) holds sc = 1/(2 sqrt N) in its imaginary part
+  static_assert(L % G == 0 || G % L == 0, "padding group");
+  static __device__ __forceinline__ int at(int j) { return j + j / G; }
+  static constexpr int LS = L + L / G;
+  static_assert(L % G == 0, "slot offsets are compile-time constants");
+  static __device__ __forceinline__ bool b_on(int s) { return SLOTS % TPP == 0 || s < SLOTS; }
+  static __device__ __forceinline__ int partner(int jj) { return jj + H * L; }
+  static __device__ __forceinline__ int unit2(int s) { return s == 0 ? H : R - s; }
+  static __device__ __forceinline__ int row1(int s) { return s; }
+  static __device__ __forceinline__ int row2(int s) { return unit2(s); }
+  static __device__ __forceinline__ int own_base(int) { return 0; }
+  static __device__ __forceinline__ int own_off(int s, int i) { return i < L ? s * LS + i + i / G : unit2(s) * LS + (i - L) + (i - L) / G; }
+
+  // a[r] = z at jj + r L, b[r] = z at jj + (r + R/2) L; on return y_k[jj] in the same order
+  static __device__ __forceinline__ void a(C (&va)[H], C (&vb)[H], int jj, const C* __restrict__ tw) {
+    C x[R];
+#pragma unroll
+    for (int r = 0; r < H; ++r) {
+      x[r] = va[r];
+      x[H + r] = vb[r];
+    }
+    Dft<T, R>::run(x);
+    va[0] = x[0];
+#pragma unroll
+    for (int k = 1; k < R; ++k) (k < H ? va[k < H ? k : 0] : vb[k < H ? 0 : k - H]) = cmul(tw[k * L + jj], x[k]);
+  }
+  static __device__ __forceinline__ void at_(C (&va)[H], C (&vb)[H], int jj, const C* __restrict__ tw) {
+    C x[R];
+    x[0] = va[0];
+#pragma unroll
+    for (int k = 1; k < R; ++k) x[k] = cmul(tw[k * L + jj], k < H ? va[k < H ? k : 0] : vb[k < H ? 0 : k - H]);
+    Dft<T, R>::run(x);
+#pragma unroll
+    for (int r = 0; r < H; ++r) {
+      va[r] = swp(x[r]);
+      vb[r] = swp(x[H + r]);
+    }
+  }
+  static __device__ __forceinline__ void a_get(const C* __restrict__ bp, int jj, C (&va)[H], C (&vb)[H]) {
+    const C* pa = bp + at(jj);
+#pragma unroll
+    for (int r = 0; r < H; ++r) {
+      va[r] = pa[r * LS];
+      vb[r] = pa[(r + H) * LS];
+    }
+  }
+  static __device__ __forceinline__ void a_put(C* __restrict__ bp, int jj, const C (&va)[H], const C (&vb)[H]) {
+    C* pa = bp + at(jj);
+#pragma unroll
+    for (int r = 0; r < H; ++r) {
+      pa[r * LS] = va[r];
+      pa[(r + H) * LS] = vb[r];
+    }
+  }
+  static __device__ __forceinline__ void b_mid(C* __restrict__, int, const C* __restrict__) {}
+  static __device__ __forceinline__ void bt_mid(C* __restrict__, int, const C* __restrict__) {}
+  // H at n and N - n from z = Z_n, w = Z_{N-n}
+  static __device__ __forceinline__ void comb(C& z, C& w, T sc) {
+    const C s = z + w, d = z - w;   // H_n = (s.x + d.y, s.y - d.x), H_{N-n} = (s.x - d.y, s.y + d.x)
+    z = sc * sub_i(s, d);
+    w = sc * add_i(s, d);
+  }
+  // transpose, components swapped
+  static __device__ __forceinline__ void comb_t(C& p, C& r, T sc) {
+    const C s = p + r, d = p - r;   // z = (s.x - d.y, s.y + d.x), w = (s.x + d.y, s.y - d.x)
+    p = sc * swp(add_i(s, d));
+    r = sc * swp(sub_i(s, d));
+  }
+  static __device__ __forceinline__ void b_end(const C* __restrict__ bp, int s, C (&z)[VB], const C* __restrict__ tw) {
+    const T sc = tw[0].y;
+    C u[L], v[L];
+    const C *pu = bp + s * LS, *pv = bp + unit2(s) * LS;
+#pragma unroll
+    for (int j = 0; j < L; ++j) {
+      u[j] = pu[j + j / G];
+      v[j] = pv[j + j / G];
+    }
+    Dft<T, L>::run(u);
+    Dft<T, L>::run(v);
+    if (s == 0) {
+      u[0] = (sc + sc) * u[0];
+      u[L / 2] = (sc + sc) * u[L / 2];
+#pragma unroll
+      for (int m = 1; m < L / 2; ++m) comb(u[m], u[L - m], sc);
+#pragma unroll
+      for (int m = 0; m < L / 2; ++m) comb(v[m], v[L - 1 - m], sc);
+    } else {
+#pragma unroll
+      for (int m = 0; m < L; ++m) comb(u[m], v[L - 1 - m], sc);
+    }
+#pragma unroll
+    for (int j = 0; j < L; ++j) {
+      z[j] = u[j];
+      z[L + j] = v[j];
+    }
+  }
+  static __device__ __forceinline__ void bt_begin(C* __restrict__ bp, int s, C (&z)[VB], const C* __restrict__ tw) {
+    const T sc = tw[0].y;
+    C u[L], v[L];
+#pragma unroll
+    for (int j = 0; j < L; ++j) {
+      u[j] = z[j];
+      v[j] = z[L + j];
+    }
+    if (s == 0) {
+      u[0] = (sc + sc) * swp(u[0]);
+      u[L / 2] = (sc + sc) * swp(u[L / 2]);
+#pragma unroll
+      for (int m = 1; m < L / 2; ++m) comb_t(u[m], u[L - m], sc);
+#pragma unroll
+      for (int m = 0; m < L / 2; ++m) comb_t(v[m], v[L - 1 - m], sc);
+    } else {
+#pragma unroll
+      for (int m = 0; m < L; ++m) comb_t(u[m], v[L - 1 - m], sc);
+    }
+    Dft<T, L>::run(u);
+    Dft<T, L>::run(v);
+    C *pu = bp + s * LS, *pv = bp + unit2(s) * LS;
+#pragma unroll
+    for (int j = 0; j < L; ++j) {
+      pu[j + j / G] = u[j];
+      pv[j + j / G] = v[j];
     }
   }
 };

@@ -1,4 +1,5 @@
-// fold_pass.cuh - the axis passes of Dirichlet plans and batches on the folded DST-I (fold_dst.cuh).
+// fold_pass.cuh - the axis passes of plans and batches on the two-step transforms of fold_dst.cuh: the folded DST-I of
+// Dirichlet axes and the Hartley transform of periodic ones.
 //
 // A CTA owns P pencil pairs (P a power of two) of one axis; thread tid works for pair tid % P as thread tid / P of
 // it. What bounds these passes is the chain load - A - exchange - B - store and, at 3D sizes, HBM; so data
@@ -23,8 +24,10 @@ namespace etd {
 // to 32 two (128 registers); FP64 plans run CTAs of at most 128 threads, up to 16 values 3 per SM and 32 values 2,
 // and from N = 768 CTAs of 256 threads with the full register file.
 // The stage kernels with weight tables (TAB: 2D plans, whose few tiles give an SM one or two CTAs) take one fewer.
-template <class T, int N, bool TAB = false> struct FoldBudget {
-  using F = Fold<T, N>;
+// PER: periodic axes (FoldH), else Dirichlet (Fold).
+template <class T, int N, bool PER> using FoldOf = typename std::conditional<PER, FoldH<T, N>, Fold<T, N>>::type;
+template <class T, int N, bool PER, bool TAB = false> struct FoldBudget {
+  using F = FoldOf<T, N, PER>;
   static constexpr int VALS = F::R > F::VB ? F::R : F::VB;
   static constexpr int THREADS = sizeof(T) == 4 || F::L == 128 ? 256 : 128;
   static constexpr int BLOCKS = sizeof(T) == 8 && F::L == 128 ? 1 : (VALS <= 16 ? 3 : 2) - (TAB ? 1 : 0);
@@ -92,9 +95,9 @@ template <class T> __device__ __forceinline__ Cx<T> phi2_pair(Cx<T> zeta, Cx<T> 
 
 // TAB: the stage weights come from the plan's per-mode tables (2D plans), else from phi evaluated per mode.
 // dense: the caller's field (ENTRY source, EXIT destination).
-template <class T, int N, int OP, bool TAB>
+template <class T, int N, bool PER, int OP, bool TAB>
 __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, T* dense) {
-  using F = Fold<T, N>;
+  using F = FoldOf<T, N, PER>;
   using C = Cx<T>;
   using VT = typename V2<T>::type;
   constexpr int H = F::H, QB = F::QB, VB = F::VB, HV = F::HV, TPP = F::TPP;
@@ -133,7 +136,7 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
       rs = (size_t)A.nx * A.ny;
       base = x0 + (long long)o * A.nx;
     }
-    if (o == 0 && A.ndim == 3) {   // boundary plane z = 0 (axis y) or row y = 0 (axis z): stays zero
+    if (!PER && o == 0 && A.ndim == 3) {   // boundary plane z = 0 (axis y) or row y = 0 (axis z): stays zero
       count_step(A);
       return;
     }
@@ -254,13 +257,15 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
       reinterpret_cast<VL*>(dst + (size_t)rb * A.nx)[k] = vb;
     }
   };
-  // dense user rows: nx - 1 interior values of the rows with y >= 1 (and z >= 1)
+  // dense user rows: nx - 1 interior values of the rows with y >= 1 (and z >= 1); periodic: the pitched rows
   auto dense_row = [&](int r) -> long long {
+    if constexpr (PER) return (long long)r * A.nx;
     const int y = r % A.ny, z = r / A.ny;
     if (y == 0 || (A.ndim == 3 && z == 0)) return -1;
     return ((A.ndim == 3 ? (long long)(z - 1) * (A.ny - 1) : 0LL) + (y - 1)) * (A.nx - 1);
   };
 
+  constexpr int X0 = PER ? 0 : 1;   // dense column of pitched index x is x - X0
   C va[H], vb[H];
   const size_t ostep = (size_t)F::STEP * rs * sizeof(T);   // bytes between a thread's consecutive rows after step B
   if constexpr (XAX) {
@@ -270,8 +275,8 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
         const long long da = q0 + pp < A.npairs ? dense_row(2 * (q0 + pp)) : -1, db = q0 + pp < A.npairs ? dense_row(2 * (q0 + pp) + 1) : -1;
         for (int x = tid; x < N; x += NT) {
           C c{T(0), T(0)};
-          if (x > 0 && da >= 0) c.x = dense[da + x - 1];
-          if (x > 0 && db >= 0) c.y = dense[db + x - 1];
+          if (x >= X0 && da >= 0) c.x = dense[da + x - X0];
+          if (x >= X0 && db >= 0) c.y = dense[db + x - X0];
           buf[pp * LP + F::at(x)] = c;
         }
       }
@@ -337,7 +342,7 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
       const int s = l + TPP * q;
       if (F::b_on(s)) {
         C z[VB];
-        F::b_end(bp, s, z);
+        F::b_end(bp, s, z, tw);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const unsigned off = ((unsigned)(h ? F::row2(s) : F::row1(s)) * (unsigned)rs + 2 * p) * (unsigned)sizeof(T);
@@ -351,7 +356,7 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
     C z[QB][VB];
 #pragma unroll
     for (int q = 0; q < QB; ++q)
-      if (F::b_on(l + TPP * q)) F::b_end(bp, l + TPP * q, z[q]);
+      if (F::b_on(l + TPP * q)) F::b_end(bp, l + TPP * q, z[q], tw);
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < QB; ++q)
@@ -369,8 +374,8 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
         const long long da = dense_row(2 * (q0 + pp)), db = dense_row(2 * (q0 + pp) + 1);
         for (int x = tid; x < N; x += NT) {
           const C c = buf[pp * LP + F::at(x)];
-          if (x > 0 && da >= 0) dense[da + x - 1] = c.x;
-          if (x > 0 && db >= 0) dense[db + x - 1] = c.y;
+          if (x >= X0 && da >= 0) dense[da + x - X0] = c.x;
+          if (x >= X0 && db >= 0) dense[db + x - X0] = c.y;
         }
       }
     } else {
@@ -418,11 +423,30 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
       C z[VB];
       [[maybe_unused]] C un[CH];
       if constexpr (STAGE && !TAB) load_u(s, 0, un);
-      F::b_end(bp, s, z);
+      F::b_end(bp, s, z, tw);
       if constexpr (OP == OP_REACT) {
         const T fl = A.flin, fc = A.fcub;
 #pragma unroll
-        for (int i = 0; i < VB; ++i) z[i] = mul2(z[i], fma2(mul2(C{fc, fc}, z[i]), z[i], C{fl, fl}));
+        for (int i = 0; i < VB; ++i) {
+          const C r = mul2(z[i], fma2(mul2(C{fc, fc}, z[i]), z[i], C{fl, fl}));
+          if constexpr (PER) {
+            // the logarithmic term of the Flory-Huggins reaction (periodic plans): through the thread's own slots below
+            if (A.flog != T(0)) bp[F::own_off(s, i)] = z[i];
+          }
+          z[i] = r;
+        }
+        if constexpr (PER) {
+          if (A.flog != T(0)) {
+            const T fg = A.flog;
+#pragma unroll 2
+            for (int i = 0; i < VB; ++i) {   // a loop: artanh's code once
+              const C w = bp[F::own_off(s, i)];
+              bp[F::own_off(s, i)] = C{fg * artanh_(w.x), fg * artanh_(w.y)};
+            }
+#pragma unroll
+            for (int i = 0; i < VB; ++i) z[i] = z[i] + bp[F::own_off(s, i)];
+          }
+        }
       } else if constexpr (TAB) {
         T* g1 = A.out1 + base;
 #pragma unroll
@@ -481,16 +505,20 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
           for (int i = 0; i < CH; ++i) {
             const C u = uc[i], w = zo[i];
             const T zj = tzr[F::STEP * i], mj = tmr[F::STEP * i];
-            // zeta = 0 only at the boundary slot, whose values are zero: kept finite there
-            const C zs0 = pz + C{zj, zj}, zeta{zs0.x > T(0) ? zs0.x : T(1), zs0.y};
-            const C rz = rcp2(zeta), p1 = mul2(fma2(C{-mj, -mj}, pm, pm + C{mj, mj}), rz);
+            // phi_1 -> 1 as zeta -> 0 (periodic mode 0; the Dirichlet boundary slot, whose values are zero); the bounds
+            // keep the reciprocal finite
+            constexpr T lo = sizeof(T) == 4 ? T(1e-30) : T(1e-290), hi = T(1) / lo;
+            const C zt = pz + C{zj, zj}, zeta{fmin(fmax(zt.x, lo), hi), fmin(fmax(zt.y, lo), hi)};
+            const C rz = rcp2(zeta), q1 = mul2(fma2(C{-mj, -mj}, pm, pm + C{mj, mj}), rz);
+            const C p1{zt.x > lo ? q1.x : T(1), zt.y > lo ? q1.y : T(1)};
             const unsigned act = __activemask();
             C o0, o1;
             if constexpr (OP == OP_S1S) {
               const T ej = ter[F::STEP * i], cj = tcr[F::STEP * i], cmj = tcmr[F::STEP * i];
               const C p2 = phi2_pair<T>(zeta, rz, p1, act);
               // c2 phi_1(-c2 zeta) = (1 - e^{-c2 zeta}) / zeta
-              const C t1 = mul2(fma2(C{-cmj, -cmj}, pcm, pcm + C{cmj, cmj}), rz);
+              const C q2 = mul2(fma2(C{-cmj, -cmj}, pcm, pcm + C{cmj, cmj}), rz);
+              const C t1{zt.x > lo ? q2.x : A.c2, zt.y > lo ? q2.y : A.c2};
               o0 = fma2(mul2(C{tau, tau}, t1), w, mul2(mul2(pc, C{cj, cj}), u));
               o1 = fma2(mul2(C{tau, tau}, fma2(C{-inv_c2, -inv_c2}, p2, p1)), w, mul2(mul2(pe, C{ej, ej}), u));
             } else if constexpr (OP == OP_RK1S) {
@@ -507,7 +535,7 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
 #pragma unroll
         for (int i = 0; i < VB; ++i) z[i] = zs[F::own_off(s, i)];
       }
-      F::bt_begin(bp, s, z);
+      F::bt_begin(bp, s, z, tw);
     }
     unit_sync();
     if constexpr (F::BIG) {
@@ -538,22 +566,22 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
   }
 }
 
-template <class T, int N, int OP, bool TAB>
-__global__ void __launch_bounds__(FoldBudget<T, N>::THREADS, FoldBudget<T, N, TAB>::BLOCKS)
+template <class T, int N, bool PER, int OP, bool TAB>
+__global__ void __launch_bounds__(FoldBudget<T, N, PER>::THREADS, FoldBudget<T, N, PER, TAB>::BLOCKS)
     fold_kernel(const PassArgs<T> A) {
-  fold_body<T, N, OP, TAB>(A, (int)blockIdx.x, OP == OP_ENTRY ? const_cast<T*>(A.in0) : A.out0);
+  fold_body<T, N, PER, OP, TAB>(A, (int)blockIdx.x, OP == OP_ENTRY ? const_cast<T*>(A.in0) : A.out0);
 }
 
 // Batches: CTA b works on tile map[b].y of problem descs[map[b].x]; entry and exit passes take the caller's field
 // from user[].
-template <class T, int N, int OP>
-__global__ void __launch_bounds__(FoldBudget<T, N>::THREADS, FoldBudget<T, N>::BLOCKS)
+template <class T, int N, bool PER, int OP>
+__global__ void __launch_bounds__(FoldBudget<T, N, PER>::THREADS, FoldBudget<T, N, PER>::BLOCKS)
     fold_kernel_batched(const PassArgs<T>* __restrict__ descs, const int2* __restrict__ map, T* const* __restrict__ user) {
   const int2 m = map[blockIdx.x];
   const PassArgs<T>& A = descs[m.x];   // read in place
   T* dense = nullptr;
   if (OP == OP_ENTRY || OP == OP_EXIT) dense = user[A.user_slot];
-  fold_body<T, N, OP, false>(A, m.y, dense);
+  fold_body<T, N, PER, OP, false>(A, m.y, dense);
 }
 
 // Shared memory of a launch: op, pairs per CTA, pair stride, tables / staged weights.
@@ -568,25 +596,25 @@ inline size_t fold_smem_bytes(const KernelInfo& k, int op, int P, int lp, bool t
   return b;
 }
 
-template <class T, int N> KernelInfo fold_info() {
-  using F = Fold<T, N>;
+template <class T, int N, bool PER> KernelInfo fold_info() {
+  using F = FoldOf<T, N, PER>;
   KernelInfo k{};
   k.N = N;
   k.tpp = F::TPP;
   k.lp = F::LP;
   k.elem = (int)sizeof(T);
-  k.fft_len = 2 * N;
-  k.odd = V_FOLD;
+  k.fft_len = PER ? N : 2 * N;
+  k.odd = PER ? V_FOLDH : V_FOLD;
   k.padg = F::G;
   k.twn = F::TWN;
   k.radix[0] = F::R;
   k.radix[1] = F::L;
-  k.min_blocks = FoldBudget<T, N>::BLOCKS;
-  k.max_threads = FoldBudget<T, N>::THREADS;
+  k.min_blocks = FoldBudget<T, N, PER>::BLOCKS;
+  k.max_threads = FoldBudget<T, N, PER>::THREADS;
   k.own_vals = F::QB * F::VB;
 #define ETD_FOLD_OP(OP)                                                                   \
-  k.fn_op[OP] = reinterpret_cast<const void*>(&fold_kernel<T, N, OP, false>);             \
-  k.fn_batched_op[OP] = reinterpret_cast<const void*>(&fold_kernel_batched<T, N, OP>);
+  k.fn_op[OP] = reinterpret_cast<const void*>(&fold_kernel<T, N, PER, OP, false>);             \
+  k.fn_batched_op[OP] = reinterpret_cast<const void*>(&fold_kernel_batched<T, N, PER, OP>);
   ETD_FOLD_OP(OP_ENTRY)
   ETD_FOLD_OP(OP_EXIT)
   ETD_FOLD_OP(OP_REACT)
@@ -595,10 +623,10 @@ template <class T, int N> KernelInfo fold_info() {
   ETD_FOLD_OP(OP_S1S)
   ETD_FOLD_OP(OP_S2S)
 #undef ETD_FOLD_OP
-  k.fn_tab[OP_RK1S] = reinterpret_cast<const void*>(&fold_kernel<T, N, OP_RK1S, true>);
-  k.fn_tab[OP_S1S] = reinterpret_cast<const void*>(&fold_kernel<T, N, OP_S1S, true>);
-  k.fn_tab[OP_S2S] = reinterpret_cast<const void*>(&fold_kernel<T, N, OP_S2S, true>);
-  k.fn_x = reinterpret_cast<const void*>(&fold_kernel<T, N, OP_TRANSFORM_X, false>);
+  k.fn_tab[OP_RK1S] = reinterpret_cast<const void*>(&fold_kernel<T, N, PER, OP_RK1S, true>);
+  k.fn_tab[OP_S1S] = reinterpret_cast<const void*>(&fold_kernel<T, N, PER, OP_S1S, true>);
+  k.fn_tab[OP_S2S] = reinterpret_cast<const void*>(&fold_kernel<T, N, PER, OP_S2S, true>);
+  k.fn_x = reinterpret_cast<const void*>(&fold_kernel<T, N, PER, OP_TRANSFORM_X, false>);
   return k;
 }
 

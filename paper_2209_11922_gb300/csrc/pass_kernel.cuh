@@ -113,23 +113,13 @@ template <> struct V2<double> { using type = double2; };
 // FP32 kernels whose transforms fit are held to 64 registers (two 512-thread CTAs per SM), so that
 // twice as many warps hide shared-memory and FMA latency; the others keep 128.
 template <class T, int N, int VAR> constexpr int pass_min_blocks();
-// Kernels compiled with the table epilogue (per-mode weight tables of FP32 2D plans): the FP32 ones with
+// Kernels compiled with the table epilogue (per-mode weight tables of 2D plans): the FP64 ones, and the FP32 ones with
 // the full register budget.
-template <class T, int N, int VAR> constexpr bool TABLES_ON() { return sizeof(T) == 4 && pass_min_blocks<T, N, VAR>() == 1; }
-// Of those, the lengths whose tile leaves room for the tile's rows of the tables in shared memory
+template <class T, int N, int VAR> constexpr bool TABLES_ON() { return sizeof(T) == 8 || pass_min_blocks<T, N, VAR>() == 1; }
+// Of those, the FP32 lengths whose tile leaves room for the tile's rows of the tables in shared memory
 // (staged before the dependency wait; the host passes no tables where a launch cannot stage them);
 // longer axes read the tables from global memory.
-template <class T, int N, int VAR> constexpr bool TABLES_STAGED() { return TABLES_ON<T, N, VAR>() && N <= 1536; }
-// Shapes with kernels per operation for the passes of a time step (REACT, TRANSFORM, RK1S, S1S, S2S): the FP32
-// length of the periodic 3D workload. (Dirichlet axes of 32 and more run the kernels of fold_pass.cuh.)
-template <class T, int N, int VAR> constexpr bool pass_op_kernels() {
-  return sizeof(T) == 4 && VAR == V_HART && N == 128;
-}
-// FP64: the operation-fixed kernels (the 2D FP64 workloads' axis length) read the tables from global memory.
-template <class T, int N, int VAR> constexpr bool TABLES_ANY() {
-  return TABLES_ON<T, N, VAR>() || (sizeof(T) == 8 && pass_op_kernels<T, N, VAR>());
-}
-
+template <class T, int N, int VAR> constexpr bool TABLES_STAGED() { return sizeof(T) == 4 && TABLES_ON<T, N, VAR>() && N <= 1536; }
 // Per-mode weights of one pencil pair at table position m: S1 four values (two per pencil), S2 and RK1
 // two (one per pencil), loaded as 16-byte vectors.
 template <class T> struct PairWeights;
@@ -163,10 +153,7 @@ template <class T> __device__ __forceinline__ void count_step(const PassArgs<T>&
   }
 }
 
-// OPC: the pass operation fixed at compile time (one of PassOp), or -1 to take it from A.op. A kernel
-// with a fixed operation holds only that operation's code, so the instructions a launch executes lie
-// together (fewer instruction-cache misses than in the kernel that serves every operation).
-template <class T, int N, int VAR, int OPC = -1>
+template <class T, int N, int VAR>
 __device__ __forceinline__ void pass_body(const PassArgs<T>& A, const int tile) {
   using L = PairLayout<T, N, VAR>;
   constexpr bool PER = L::HART;   // periodic: no boundary planes, rows or slots
@@ -181,7 +168,7 @@ __device__ __forceinline__ void pass_body(const PassArgs<T>& A, const int tile) 
   const C* __restrict__ tw = tws;
   const T* __restrict__ sn = A.sn;
   C* b0 = tws + ((TWN + 1) & ~1);
-  const int op = OPC >= 0 ? OPC : A.op;
+  const int op = A.op;
   const bool two = (op == OP_RK1 || op == OP_S1 || op == OP_S2 || op == OP_RK1S || op == OP_S1S || op == OP_S2S);
   C* b1 = b0 + A.P * LP;
   C* scr = b0 + (two ? 2 : 1) * A.P * LP;
@@ -494,9 +481,8 @@ __device__ __forceinline__ void pass_body(const PassArgs<T>& A, const int tile) 
   // values (FP32 plans: rounded once) (A.coef, [y mode][x mode]; e^{-z}, e^{-c2 z} are products of the
   // per-axis factors), with every table load of a chunk of positions issued before the first use. Same
   // effect on the buffers as the epilogue above.
-  // Compiled into the FP32 kernels with the full register budget and the FP64 operation-fixed kernels
-  // only; the others evaluate the weights.
-  constexpr bool TABLES = TABLES_ANY<T, N, VAR>();
+  // The FP32 kernels with the halved register budget evaluate the weights.
+  constexpr bool TABLES = TABLES_ON<T, N, VAR>();
   auto table_epilogue = [&](int kind, C* bpk) {
     if constexpr (TABLES) {
       constexpr int CNT = (N + TPP - 1) / TPP, CH = sizeof(T) == 4 ? 4 : 2;
@@ -621,12 +607,6 @@ __global__ void __launch_bounds__(512, pass_min_blocks<T, N, VAR>()) pass_kernel
   pass_body<T, N, VAR>(A, (int)blockIdx.x);
 }
 
-// The same with the operation fixed (A.op must equal OPC).
-template <class T, int N, int VAR, int OPC>
-__global__ void __launch_bounds__(512, pass_min_blocks<T, N, VAR>()) pass_kernel_op(const PassArgs<T> A) {
-  pass_body<T, N, VAR, OPC>(A, (int)blockIdx.x);
-}
-
 // Batches: one launch covers the tiles of many independent problems whose transformed axis has
 // length N. CTA b works on tile map[b].y of the problem described by descs[map[b].x]; entry and exit
 // passes take the caller's field pointer from user[descs[.].user_slot].
@@ -642,33 +622,23 @@ __global__ void __launch_bounds__(512, pass_min_blocks<T, N, VAR>())
   pass_body<T, N, VAR>(A, m.y);
 }
 
-// The same with the operation fixed (every descriptor's op must equal OPC).
-template <class T, int N, int VAR, int OPC>
-__global__ void __launch_bounds__(512, pass_min_blocks<T, N, VAR>())
-    pass_kernel_batched_op(const PassArgs<T>* __restrict__ descs, const int2* __restrict__ map, T* const* __restrict__) {
-  const int2 m = map[blockIdx.x];
-  // the descriptor is read in place (read-only global memory, reloaded where needed) rather than copied
-  // into registers, which the stage passes cannot spare
-  pass_body<T, N, VAR, OPC>(descs[m.x], m.y);
-}
-
 // Host-side description of one instantiation.
 struct KernelInfo {
   const void* fn;
   const void* fn_batched;
-  const void* fn_op[OP_COUNT];           // kernels with the operation fixed, by PassOp (NULL: use fn)
-  const void* fn_batched_op[OP_COUNT];   // the same for batches (NULL: use fn_batched)
+  const void* fn_op[OP_COUNT];           // kernels of one operation each, by PassOp (two-step kernels)
+  const void* fn_batched_op[OP_COUNT];   // the same for batches
   int N;
   int tpp;
   int lp;
   int elem;   // sizeof(T)
   int fft_len;  // M: 2N (odd extension) or N (recurrence, Hartley)
-  int odd;      // transform variant: V_ODD odd extension, V_REC recurrence, V_HART Hartley
+  int odd;      // transform variant (enum Variant)
   int padg;     // one padding slot every padg positions
   int twn;      // twiddle table entries
   int radix[4]; // Stockham radices (0-terminated)
   int min_blocks;  // CTAs per SM the register budget was compiled for
-  // folded-odd-extension kernels (odd == V_FOLD: fn_op and fn_batched_op only)
+  // two-step kernels (V_FOLD, V_FOLDH: fn_op and fn_batched_op only)
   const void* fn_tab[OP_COUNT];  // stage passes reading per-mode weight tables
   const void* fn_x;              // OP_TRANSFORM along x
   int max_threads;               // CTA size limit
@@ -688,21 +658,6 @@ template <class T, int N, int VAR> KernelInfo kernel_info() {
                {},
                N, L::TPP, L::LP, (int)sizeof(T), L::M,
                VAR, L::PADG, L::TWN, {0, 0, 0, 0}, pass_min_blocks<T, N, VAR>()};
-  if constexpr (pass_op_kernels<T, N, VAR>()) {
-    // single plans run the stage passes on the spectral state (RK1S, S1S, S2S)
-    k.fn_op[OP_REACT] = reinterpret_cast<const void*>(&pass_kernel_op<T, N, VAR, OP_REACT>);
-    k.fn_op[OP_TRANSFORM] = reinterpret_cast<const void*>(&pass_kernel_op<T, N, VAR, OP_TRANSFORM>);
-    k.fn_op[OP_RK1S] = reinterpret_cast<const void*>(&pass_kernel_op<T, N, VAR, OP_RK1S>);
-    k.fn_op[OP_S1S] = reinterpret_cast<const void*>(&pass_kernel_op<T, N, VAR, OP_S1S>);
-    k.fn_op[OP_S2S] = reinterpret_cast<const void*>(&pass_kernel_op<T, N, VAR, OP_S2S>);
-    // batches (FP32) are 2D: TRANSFORM only at entry (the generic kernel)
-    if constexpr (sizeof(T) == 4) {
-    k.fn_batched_op[OP_REACT] = reinterpret_cast<const void*>(&pass_kernel_batched_op<T, N, VAR, OP_REACT>);
-    k.fn_batched_op[OP_RK1S] = reinterpret_cast<const void*>(&pass_kernel_batched_op<T, N, VAR, OP_RK1S>);
-    k.fn_batched_op[OP_S1S] = reinterpret_cast<const void*>(&pass_kernel_batched_op<T, N, VAR, OP_S1S>);
-    k.fn_batched_op[OP_S2S] = reinterpret_cast<const void*>(&pass_kernel_batched_op<T, N, VAR, OP_S2S>);
-    }
-  }
   radix_list(k.radix, typename L::Plan::R{});
   return k;
 }
