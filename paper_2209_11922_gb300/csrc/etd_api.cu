@@ -92,6 +92,7 @@ struct Launch {
                                                                                 : sizeof(GemmParams)];
   size_t args_size;
   double alg_bytes;  // algorithmic HBM bytes of this launch (fields read + written)
+  bool pdl = true;   // programmatic dependent launch (choose_pdl)
 };
 
 int env_int(const char* name, int dflt) {
@@ -490,10 +491,32 @@ etd_status launch(const Launch& L, cudaStream_t s) {
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = use_pdl ? 1 : 0;
+  cfg.numAttrs = use_pdl && L.pdl ? 1 : 0;
   cudaError_t e = cudaLaunchKernelExC(&cfg, L.fn, argv);
   if (e != cudaSuccess) return fail(ETD_ERR_CUDA, "kernel launch: %s", cudaGetErrorString(e));
   return ETD_OK;
+}
+
+// Which launches of a time step take programmatic dependent launch. It hides a launch's latency (2 to 4 us of a step),
+// but CTAs that start while their predecessor drains go to the SMs it leaves free, several to one SM, and stay there:
+// where the grid is a few large CTAs per SM the pass then takes as long as the SM with the most (1023^2 FP64 ETDRK1,
+// 128 CTAs: 298 us per step against 216; FP32 ETDRK2 31.9 against 28.7). So a launch goes without when it and its
+// predecessor do not fit on distinct SMs, its CTAs are large enough to load an SM (256 threads; FP64, whose units a
+// warp keeps for 64 cycles, 64), more of them fit on an SM than an even spread puts there, and there are too few of them
+// for the imbalance to average out.
+void choose_pdl(std::vector<Launch>& step, int num_sms, int elem) {
+  for (size_t i = 0; i < step.size(); ++i) {
+    Launch& L = step[i];
+    const long long grid = L.grid.x, prev = step[i ? i - 1 : step.size() - 1].grid.x;
+    const int threads = (int)L.block.x;
+    int occ = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, L.fn, threads, L.smem) != cudaSuccess) {
+      cudaGetLastError();
+      continue;
+    }
+    L.pdl = !(grid + prev > num_sms && grid < 4LL * num_sms && threads >= (elem == 8 ? 64 : 256) &&
+              occ > (grid + num_sms - 1) / num_sms);
+  }
 }
 
 // Sets the source fields of the step's launches: the reaction passes (stage 1 at t_n, stage 2 at
@@ -644,6 +667,7 @@ etd_status build_step(etd_plan_s* pl) {
   }
 #undef BND
 #undef ADD
+  choose_pdl(pl->step, pl->num_sms, pl->elem);
   return ETD_OK;
 }
 
