@@ -32,6 +32,7 @@
 
 #include "../../include/etd.h"
 #include "boundary.cuh"
+#include "dense_pass.cuh"
 #include "fold_pass.cuh"
 #include "gemm_pass.cuh"
 #include "monitor.cuh"
@@ -105,7 +106,18 @@ int env_int(const char* name, int dflt) {
 // extension, which is exact in the same sense as both DST-I forms below and does less work than either, and
 // the lengths it has no plan for (below 32, 24 included) the odd extension or the recurrence: FP32 as the route
 // says (AUTO: the recurrence), FP64 the recurrence.
-int dst_variant(const etd_options& o, int64_t n, int64_t pairs) {
+// FP64 single plans (`batch` false) over few short pencils take dense products: they cost pencils n^2 / 608 cycles
+// per transform where an FFT pass costs its longest thread, 16 to 60 thousand cycles at these lengths. The lines lie
+// where the two were equal (us per ETDRK2 step, dense against FFT: 64^2 19.5 / 138, 128^2 35 / 157, 256^2 148 / 173,
+// 48^3 108 / 251; 64^3 259 / 232 by the recurrence, 96^3 ETDRK1 490 / 271).
+int dst_variant(const etd_options& o, int64_t n, int64_t pairs, bool batch) {
+  if (o.dtype == ETD_F64 && !batch) {
+    if (n <= 256 && 2 * pairs * n * n <= (n == 64 ? 12000000 : 20000000)) return V_DENSE;
+    // N = 64 up to 4000 pairs, where the folded plan's 4 threads per pair leave schedulers idle, and N = 1536 and 2048
+    // over few pencils: the recurrence's threads hold half the values (8, and 16 against 24 and 32; 64^3 286 us by the
+    // folded plan, 2048 x 64 222 against 307)
+    if (o.bc == ETD_BC_DIRICHLET && ((n == 64 && pairs <= 4000) || ((n == 1536 || n == 2048) && pairs <= 128))) return V_REC;
+  }
   if (o.bc == ETD_BC_PERIODIC) return foldh_has(o.dtype == ETD_F32 ? 4 : 8, (int)n, pairs) ? V_FOLDH : V_HART;
   if (fold_has((int)n)) return V_FOLD;
   return o.dtype == ETD_F32 && o.route == ETD_ROUTE_FFT ? V_ODD : V_REC;
@@ -302,26 +314,54 @@ __global__ void __launch_bounds__(256) pack_kernel(const PassArgs<T> A) {
 template <class T>
 etd_status make_fold_launch(etd_plan_s* pl, const KernelInfo* k, PassArgs<T>& a, int kind, double fields_rw, Launch& L) {
   const int op = a.op;
+  const int sms = pl->num_sms;
   int P = 16;
   while (P * k->tpp > k->max_threads) P /= 2;
   long long grid = 0;
   int optin = 0;
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, pl->device);
   const bool tab = fold_is_stage(op) && a.coef;
+  // Pairs per CTA: at most 16 (128-byte FP32 row segments); fewer where that leaves fewer than two CTAs per SM, but
+  // whole warps (an FP64 instruction holds its scheduler for 64 cycles whatever its lanes do: 24 x 256 x 64 FP64 with
+  // half-warp CTAs took 1.6 times as long), and on strided axes rows of at least one 32-byte sector.
+  const long long pairs = (long long)pl->nfield / k->N / 2;
+  const bool big = k->radix[1] >= 64;
+  int pmin = 32 / k->tpp > 1 ? 32 / k->tpp : 1;
+  if (a.axis != 0 && pmin < 16 / (int)sizeof(T)) pmin = 16 / (int)sizeof(T);
+  if (big) {
+    // Units of UT threads: with 32 / UT pairs unit 0 of step B, which runs other code, is a warp of its own; with fewer
+    // it is part of one, which then runs both. Along x the choice minimises the pairs on the busiest SM times that
+    // cost; strided axes keep their sectors (48 x 1024 FP32 took 220 us at one pair against 186 at four).
+    const int whole = k->radix[1] == 256 ? 2 : 4;   // 32 / UT
+    int pick = whole;
+    double best = 1e30;
+    for (int q = whole; q >= 1 && a.axis == 0; q /= 2) {
+      const double cost = (double)((pairs / q + sms - 1) / sms * q) * (q == whole ? 1.0 : 2 * q == whole ? 1.3 : 1.6);
+      if (cost < best) {
+        best = cost;
+        pick = q;
+      }
+    }
+    if (a.axis == 0 || pick > pmin) pmin = pick;
+  }
   if (a.axis == 0) {
-    a.npairs = pl->ny * pl->nz / 2;
-    // Where step B's units are 8 threads (L >= 64) four pairs: unit 0 of step B, which runs other code, is then a warp of its
-    // own instead of a part of one.
-    const int pmin = k->radix[1] >= 64 ? 4 : 1;
-    while (P > pmin && (a.npairs + P - 1) / P < 2 * pl->num_sms) P /= 2;
-    grid = (a.npairs + P - 1) / P;
+    while (P > pmin && pairs / P < 2 * sms) P /= 2;
+    a.npairs = (int)pairs;
+    grid = (pairs + P - 1) / P;
   } else {
-    // A tile's row segment (2P values) is at least one 32-byte sector
+    // tile widths 2 P divide the x extent: powers of two, and in FP64 12, 6 and 3 pairs for extents such as 24
     const int other = (a.axis == 1) ? pl->nz : pl->ny;
-    const int pmin = k->radix[1] >= 64 ? 4 : 16 / (int)sizeof(T);
-    while (P > pmin && (pl->nx / (2 * P)) * (long long)other < 2 * pl->num_sms) P /= 2;
-    while (P > 1 && (pl->nx % (2 * P) != 0 || fold_smem_bytes(*k, op, P, pair_stride(*k, P), tab, false) > (size_t)optin)) P /= 2;
-    if (pl->nx % (2 * P) != 0) return fail(ETD_ERR_UNSUPPORTED, "x extent %d not even", pl->nx);
+    static const int cand[] = {16, 12, 8, 6, 4, 3, 2, 1};
+    int pick = 0;
+    for (int q : cand) {
+      if (pl->nx % (2 * q) != 0 || q * k->tpp > k->max_threads || ((q & (q - 1)) && (sizeof(T) == 4 || pl->nx % 16 == 0))) continue;
+      if (fold_smem_bytes(*k, op, q, pair_stride(*k, q), tab, false) > (size_t)optin) continue;
+      if (pick && q < pmin) break;
+      pick = q;
+      if (pairs / q >= 2 * sms) break;
+    }
+    if (!pick) return fail(ETD_ERR_UNSUPPORTED, "x extent %d not even", pl->nx);
+    P = pick;
     a.tiles_x = pl->nx / (2 * P);
     grid = (long long)a.tiles_x * other;
   }
@@ -348,6 +388,41 @@ etd_status make_fold_launch(etd_plan_s* pl, const KernelInfo* k, PassArgs<T>& a,
   return ETD_OK;
 }
 
+// One pass by dense products (dense_pass.cuh, FP64).
+etd_status make_dense_launch(etd_plan_s* pl, PassArgs<double>& a, int kind, double fields_rw, Launch& L) {
+  static_assert(sizeof(DenseArgs) <= sizeof(Launch::args), "launch argument buffer too small");
+  DenseArgs g;
+  const int N = (int)pl->N[a.axis], op = a.op;
+  const long long pencils = (long long)pl->nfield / N;
+  g.N = N;
+  g.per = pl->periodic ? 1 : 0;
+  // threads per output: enough to give each of the chip's 4 x num_sms schedulers a warp
+  const long long want = 32LL * 4 * pl->num_sms;
+  g.KS = 1;
+  while (g.KS < 4 && (long long)pl->nfield * g.KS < want && 2 * g.KS * N <= 512) g.KS *= 2;
+  int W = 4;
+  while (W > 1 && (W * N * g.KS > 256 || (a.axis != 0 && pl->nx % W != 0))) W /= 2;
+  a.P = W;
+  long long grid;
+  if (a.axis == 0) {
+    grid = (pencils + W - 1) / W;
+  } else {
+    a.tiles_x = pl->nx / W;
+    grid = (long long)a.tiles_x * (a.axis == 1 ? pl->nz : pl->ny);
+  }
+  g.a = a;
+  L.fn = find_dense_kernel(op == OP_TRANSFORM && a.axis == 0 ? OP_TRANSFORM_X : op);
+  if (!L.fn) return fail(ETD_ERR_UNSUPPORTED, "no dense kernel for pass %d", op);
+  L.grid = dim3((unsigned)grid);
+  L.block = dim3((unsigned)(W * N * g.KS));
+  L.smem = dense_smem_bytes(N, W, g.KS);
+  L.kind = kind;
+  memcpy(L.args, &g, sizeof(g));
+  L.args_size = sizeof(g);
+  L.alg_bytes = fields_rw * (double)pl->unknowns * sizeof(double);
+  return ETD_OK;
+}
+
 template <class T>
 etd_status make_launch(etd_plan_s* pl, int op, int axis, const void* in0, const void* in1, void* out0,
                        void* out1, int kind, double fields_rw, Launch& L) {
@@ -358,8 +433,9 @@ etd_status make_launch(etd_plan_s* pl, int op, int axis, const void* in0, const 
       return make_split_launch(pl, op, axis, in0, in1, out0, out1, kind, fields_rw, L);
   }
   const int N = (int)pl->N[axis];
-  const KernelInfo* k = find_pass_kernel((int)sizeof(T), N, pl->odd[axis]);
-  if (!k) return fail(ETD_ERR_UNSUPPORTED, "no kernel for axis length %d", N);
+  const bool dense = pl->odd[axis] == V_DENSE;
+  const KernelInfo* k = dense ? nullptr : find_pass_kernel((int)sizeof(T), N, pl->odd[axis]);
+  if (!k && !dense) return fail(ETD_ERR_UNSUPPORTED, "no kernel for axis length %d", N);
   PassArgs<T> a;
   fill_common<T>(pl, a);
   if (op == OP_PACK || op == OP_UNPACK) {
@@ -392,6 +468,9 @@ etd_status make_launch(etd_plan_s* pl, int op, int axis, const void* in0, const 
     if (op == OP_S1 || op == OP_S1S) a.coef = cf + pl->coef_s1;
     else if (op == OP_S2 || op == OP_S2S) a.coef = cf + pl->coef_s2;
     else if (op == OP_RK1 || op == OP_RK1S) a.coef = cf + pl->coef_rk1;
+  }
+  if constexpr (sizeof(T) == 8) {
+    if (dense) return make_dense_launch(pl, a, kind, fields_rw, L);
   }
   if (two_step(*k)) return make_fold_launch<T>(pl, k, a, kind, fields_rw, L);
   const bool two = (op == OP_RK1 || op == OP_S1 || op == OP_S2 || op == OP_RK1S || op == OP_S1S || op == OP_S2S);
@@ -502,7 +581,7 @@ etd_status launch(const Launch& L, cudaStream_t s) {
 // where the grid is a few large CTAs per SM the pass then takes as long as the SM with the most (1023^2 FP64 ETDRK1,
 // 128 CTAs: 298 us per step against 216; FP32 ETDRK2 31.9 against 28.7). So a launch goes without when it and its
 // predecessor do not fit on distinct SMs, its CTAs are large enough to load an SM (256 threads; FP64, whose units a
-// warp keeps for 64 cycles, 64), more of them fit on an SM than an even spread puts there, and there are too few of them
+// warp keeps for 64 cycles, 48: 24 x 256 x 64 ETDRK1 293 us per step against 183), more of them fit on an SM than an even spread puts there, and there are too few of them
 // for the imbalance to average out.
 void choose_pdl(std::vector<Launch>& step, int num_sms, int elem) {
   for (size_t i = 0; i < step.size(); ++i) {
@@ -514,7 +593,7 @@ void choose_pdl(std::vector<Launch>& step, int num_sms, int elem) {
       cudaGetLastError();
       continue;
     }
-    L.pdl = !(grid + prev > num_sms && grid < 4LL * num_sms && threads >= (elem == 8 ? 64 : 256) &&
+    L.pdl = !(grid + prev > num_sms && grid < 4LL * num_sms && threads >= (elem == 8 ? 48 : 256) &&
               occ > (grid + num_sms - 1) / num_sms);
   }
 }
@@ -975,7 +1054,7 @@ etd_status entry_exit_any(etd_plan_s* pl, bool entry, void* u, std::vector<Launc
 }
 
 // Tables of a folded axis (fold_dst.cuh), FP64 values rounded once to T: step A's [R/2][L/2] entries, and for
-// L >= 64 the twiddles exp(2 pi i t i / L) as [L/8][8] and the inner transform's step A entries (R = 16, L/8).
+// L >= 64 the twiddles exp(2 pi i t i / L) as [L/UT][UT] and the inner transform's step A entries (R = 2 UT, L/UT).
 template <class T>
 void append_fold_twiddles(const KernelInfo* k, std::vector<T>& h) {
   const double sc = 0.5 * sqrt(2.0 / (double)k->N);
@@ -1005,9 +1084,10 @@ void append_fold_twiddles(const KernelInfo* k, std::vector<T>& h) {
   }
   step_a(R, Ls);
   if (Ls >= 64) {
-    for (int i = 0; i < Ls / 8; ++i)
-      for (int t = 0; t < 8; ++t) put(cos(2.0 * M_PI * t * i / Ls), sin(2.0 * M_PI * t * i / Ls));
-    step_a(16, Ls / 8);
+    const int ut = Ls == 256 ? 16 : 8;   // Fold::UT
+    for (int i = 0; i < Ls / ut; ++i)
+      for (int t = 0; t < ut; ++t) put(cos(2.0 * M_PI * t * i / Ls), sin(2.0 * M_PI * t * i / Ls));
+    step_a(2 * ut, Ls / ut);
   }
 }
 
@@ -1026,6 +1106,18 @@ void append_axis_tables(const KernelInfo* k, int n, double hh, double tauD, doub
   size_t t = 0;
   if (two_step(*k)) {
     append_fold_twiddles<T>(k, h);
+    t = 1;
+  } else if (k->odd == V_DENSE) {   // the matrix of dense_pass.cuh
+    std::vector<double> sn(2 * (size_t)n), cs(2 * (size_t)n);   // at pi m / n
+    for (int m = 0; m < 2 * n; ++m) {
+      sn[m] = sin(M_PI * (double)m / (double)n);
+      cs[m] = cos(M_PI * (double)m / (double)n);
+    }
+    const double s = periodic ? 1.0 / sqrt((double)n) : sqrt(2.0 / (double)n);
+    for (int j = 0; j <= n / 2; ++j)
+      for (int q = 0; q < n; ++q)
+        h.push_back((T)(s * (periodic ? (q <= n / 2 ? cs[2 * j * q % (2 * n)] : sn[2 * j * (n - q) % (2 * n)])
+                                      : sn[j * q % (2 * n)])));
     t = 1;
   }
   for (int i = 0; !two_step(*k) && i < 4 && k->radix[i]; ++i) {
@@ -1171,7 +1263,9 @@ etd_status upload_tables(etd_plan_s* pl) {
   std::vector<T> h;
   size_t offs[3][7], soff[3] = {0, 0, 0};
   for (int a = 0; a < pl->ndim; ++a) {
-    const KernelInfo* k = find_pass_kernel((int)sizeof(T), (int)pl->N[a], pl->odd[a]);
+    KernelInfo dense{};
+    dense.odd = V_DENSE;
+    const KernelInfo* k = pl->odd[a] == V_DENSE ? &dense : find_pass_kernel((int)sizeof(T), (int)pl->N[a], pl->odd[a]);
     if (!k) return fail(ETD_ERR_UNSUPPORTED, "no kernel for axis length %lld", (long long)pl->N[a]);
     append_axis_tables<T>(k, (int)pl->N[a], pl->h[a], pl->tau * pl->D, pl->opt.c2, h, offs[a], pl->periodic != 0);
     if (pl->split[a]) soff[a] = append_split_tables<T>(h);
@@ -1841,7 +1935,7 @@ etd_status etd_plan_create(etd_plan* out, int ndim, const int64_t* N, const doub
   pl->opt = o;
   pl->elem = (o.dtype == ETD_F32) ? 4 : 8;
   for (int a = 0; a < ndim; ++a) {
-    pl->odd[a] = dst_variant(o, N[a], N[0] * N[1] * (ndim == 3 ? N[2] : 1) / N[a] / 2);
+    pl->odd[a] = dst_variant(o, N[a], N[0] * N[1] * (ndim == 3 ? N[2] : 1) / N[a] / 2, false);
   }
   // ETD_ROUTE_FFT_SPLIT: FP32 Dirichlet axes of length 1024 take the split-radix kernels (the strided
   // passes need an x extent that is a multiple of 4); every other axis the AUTO choice.
@@ -2252,8 +2346,8 @@ etd_status etd_batch_create(etd_batch* out, int count, const int64_t* N, const d
     b->hx.push_back(h[2 * i]);
     b->hy.push_back(h[2 * i + 1]);
     b->Dv.push_back(D[i]);
-    b->oddx.push_back(dst_variant(o, N[2 * i], 1024));   // the group's pairs of all problems fill the GPU
-    b->oddy.push_back(dst_variant(o, N[2 * i + 1], 1024));
+    b->oddx.push_back(dst_variant(o, N[2 * i], 1024, true));   // the group's pairs of all problems fill the GPU
+    b->oddy.push_back(dst_variant(o, N[2 * i + 1], 1024, true));
   }
   if (cudaGetDevice(&b->device) != cudaSuccess) {
     delete b;

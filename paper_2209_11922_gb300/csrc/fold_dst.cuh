@@ -15,7 +15,7 @@
 //   length L of the folded sequence d_jj = (X_0 + X_{R/2})/2, d_{L-jj} = (X_{R/2} - X_0)/2. It is computed by
 //   a DFT of the same length L (the half-length recurrence of dst_engine.cuh: y_jj = sin(pi jj/L) X_{R/2} +
 //   X_0/2, y_{L-jj} = sin(pi jj/L) X_{R/2} - X_0/2, even outputs as differences, odd ones as running sums of
-//   at most L/2 = 16 terms held by one thread), or for L = 64 and 128 by this scheme itself (R' = 16, L' = L/8).
+//   at most L/2 = 16 terms held by one thread), or for L >= 64 by this scheme itself (R' = 2 UT, L' = L/UT below).
 //   Butterflies 0 and L/2 (self-symmetric, half the data each) share one radix-R DFT: C = X^{(0)} + X^{(L/2)},
 //   from which y_k[0] = (-i sc/2)(C_k - C_{-k}) - (sc/2) cot(pi k/R)(C_k + C_{-k}) and
 //   y_k[L/2] = sc/(2 sin(pi k/R)) (C_k + C_{-k}).
@@ -34,7 +34,8 @@
 namespace etd {
 
 // Plans: radix R, sub-length L (R L = 2N), threads per pencil pair, values per thread at most R or L.
-// L <= 32: step B is one register DFT per unit. L = 64, 128: units of 8 threads, L/8 values each (L/8 x 8).
+// L <= 32: step B is one register DFT per unit. L = 64, 128: units of UT = 8 threads, L/8 values each (L/8 x 8);
+// L = 256: units of 16 threads (16 x 16).
 // G: one padding slot every G positions (G divides L, so slot offsets are compile-time constants).
 template <class T, int N> struct FoldPlan { static constexpr int R = 0, L = 0, TPP = 1, G = 1; };
 #define ETD_FOLD(NN, R_, L_, TPP_, G_)                                             \
@@ -54,7 +55,7 @@ ETD_FOLD(512, 32, 32, 16, 16)
 ETD_FOLD(768, 12, 128, 64, 8)
 ETD_FOLD(1024, 16, 128, 64, 8)
 ETD_FOLD(1536, 24, 128, 64, 8)
-ETD_FOLD(2048, 32, 128, 64, 8)
+ETD_FOLD(2048, 16, 256, 128, 16)
 #undef ETD_FOLD
 // FP64, 192..512: GB300 issues a warp's FP64 instruction over 64 cycles of one of the SM's four schedulers, whatever
 // lanes it has, so a pass over few pencils costs its longest thread: fewer values per thread and more threads
@@ -69,6 +70,7 @@ ETD_FOLD64(192, 6, 64, 32, 8)
 ETD_FOLD64(256, 8, 64, 32, 8)
 ETD_FOLD64(384, 12, 64, 32, 8)
 ETD_FOLD64(512, 16, 64, 32, 8)
+ETD_FOLD64(2048, 32, 128, 64, 8)   // R = 16, L = 256 on 128 threads: 2048 x 1024 ETDRK2 1016 us per step against 891
 #undef ETD_FOLD64
 
 constexpr bool fold_has(int n) {
@@ -241,15 +243,16 @@ template <class T, int N> struct Fold {
   static constexpr int R = Plan::R, L = Plan::L, TPP = Plan::TPP, G = Plan::G;
   static constexpr int H = R / 2;                       // units of step B
   static constexpr int UA = L / 2;                      // units of step A
-  static constexpr bool BIG = L >= 64;                 // step B across 8 threads per unit
+  static constexpr bool BIG = L >= 64;                  // step B across UT threads per unit
+  static constexpr int UT = L == 256 ? 16 : 8;
   static constexpr int QA = (UA + TPP - 1) / TPP;       // A units per thread
-  static constexpr int SLOTS = BIG ? 8 * H : H;         // thread slots of step B
+  static constexpr int SLOTS = BIG ? UT * H : H;         // thread slots of step B
   static constexpr int QB = (SLOTS + TPP - 1) / TPP;    // B slots per thread
-  static constexpr int VB = BIG ? L / 8 : L;               // values per B slot
+  static constexpr int VB = BIG ? L / UT : L;               // values per B slot
   static constexpr int LP = N + N / G;                  // complex slots per pair
-  static constexpr int UI = BIG ? VB / 2 : 1;           // A units of unit 0's inner transform (R' = 16, L' = VB)
-  // tables: A twiddles [H][UA]; BIG: exp(2 pi i t i / L) [VB][8], then unit 0's A twiddles [8][UI]
-  static constexpr int TW_A = H * UA, TW_B = BIG ? 8 * VB : 0, TW_S = BIG ? 8 * UI : 0;
+  static constexpr int UI = BIG ? VB / 2 : 1;           // A units of unit 0's inner transform (R' = 2 UT, L' = VB)
+  // tables: A twiddles [H][UA]; BIG: exp(2 pi i t i / L) [VB][UT], then unit 0's A twiddles [UT][UI]
+  static constexpr int TW_A = H * UA, TW_B = BIG ? UT * VB : 0, TW_S = BIG ? UT * UI : 0;
   static constexpr int TWN = TW_A + TW_B + TW_S;
   static_assert(L % G == 0, "padding group divides L");
   static __device__ __forceinline__ int at(int j) { return j + j / G; }
@@ -286,45 +289,45 @@ template <class T, int N> struct Fold {
 
   // Rows (output positions) of the values of B slot s: value i < HV at row1(s) + i STEP, value HV + i at
   // row2(s) + i STEP.
-  static constexpr int HV = VB / 2, STEP = BIG ? 8 * R : R;
+  static constexpr int HV = VB / 2, STEP = BIG ? UT * R : R;
   static __device__ __forceinline__ int row1(int s) {
     if constexpr (!BIG) return s;
-    const int k = s >> 3, t = s & 7;
+    const int k = s / UT, t = s % UT;
     return k == 0 ? H * t : R * t + k;
   }
   static __device__ __forceinline__ int row2(int s) {
     if constexpr (!BIG) return s == 0 ? H : R - s;
-    const int k = s >> 3, t = s & 7;
-    return k == 0 ? H * (t == 0 ? 8 : 16 - t) : R * (7 - t) + R - k;   // unit 0: the inner transform's rows
+    const int k = s / UT, t = s % UT;
+    return k == 0 ? H * (t == 0 ? UT : 2 * UT - t) : R * (UT - 1 - t) + R - k;   // unit 0: the inner transform's rows
   }
 
   // The slots b_end reads and bt_begin writes for value i: own_base(s) + own_off(i).
   static __device__ __forceinline__ int own_base(int s) {
     if constexpr (!BIG) return s * LS;
-    else return (s >> 3) == 0 ? at(VB * (s & 7)) : (s >> 3) * LS + at(8 * (s & 7));
+    else return (s / UT) == 0 ? at(VB * (s % UT)) : (s / UT) * LS + at(UT * (s % UT));
   }
   static __device__ __forceinline__ int own_off(int s, int i) {
     if constexpr (!BIG) return i + i / G;
-    else return (s >> 3) == 0 ? i + i / G : (i & 7) + (i >> 3) * (64 + 64 / G);
+    else return (s / UT) == 0 ? i + i / G : (i % UT) + (i / UT) * (UT * UT + UT * UT / G);
   }
 
   // Step B: slot s of the pair, values to registers in the order of row1 / row2. The BIG form has an exchange
   // inside its unit: mid() is the part before it.
   static __device__ __forceinline__ void b_mid(C* __restrict__ bp, int s, const C* __restrict__ tw) {
     if constexpr (BIG) {
-      const int k = s >> 3, t = s & 7;
+      const int k = s / UT, t = s % UT;
       if (k == 0) {
         if (t < UI) {
-          C va[8], vb[8];
+          C va[UT], vb[UT];
           const int part = t == 0 ? VB / 2 : VB - t;
 #pragma unroll
-          for (int r = 0; r < 8; ++r) {
+          for (int r = 0; r < UT; ++r) {
             va[r] = bp[at(VB * r + t)];
             vb[r] = bp[at(VB * r + part)];
           }
-          fold_a<T, 16, true, UI>(va, vb, t, tw + TW_A + TW_B);
+          fold_a<T, 2 * UT, true, UI>(va, vb, t, tw + TW_A + TW_B);
 #pragma unroll
-          for (int r = 0; r < 8; ++r) {
+          for (int r = 0; r < UT; ++r) {
             bp[at(VB * r + t)] = va[r];
             bp[at(VB * r + part)] = vb[r];
           }
@@ -333,11 +336,11 @@ template <class T, int N> struct Fold {
         C* p = bp + k * LS + at(t);
         C x[VB];
 #pragma unroll
-        for (int i = 0; i < VB; ++i) x[i] = p[i * (8 + 8 / G)];
+        for (int i = 0; i < VB; ++i) x[i] = p[i * (UT + UT / G)];
         Dft<T, VB>::run(x);
         const C* w = tw + TW_A + t;
 #pragma unroll
-        for (int i = 0; i < VB; ++i) p[i * (8 + 8 / G)] = i == 0 ? x[0] : cmul(w[8 * i], x[i]);
+        for (int i = 0; i < VB; ++i) p[i * (UT + UT / G)] = i == 0 ? x[0] : cmul(w[UT * i], x[i]);
       }
     }
   }
@@ -348,7 +351,7 @@ template <class T, int N> struct Fold {
       for (int j = 0; j < L; ++j) z[j] = p[j + j / G];
       fold_b<T, L>(z, s == 0);
     } else {
-      const int k = s >> 3, t = s & 7;
+      const int k = s / UT, t = s % UT;
       if (k == 0) {
         const C* p = bp + at(VB * t);
 #pragma unroll
@@ -356,16 +359,16 @@ template <class T, int N> struct Fold {
         fold_b<T, VB>(z, t == 0);
       } else {
 #pragma unroll
-        for (int h = 0; h < VB / 8; ++h) {
-          const C* p = bp + k * LS + at(8 * (t + 8 * h));
-          C x[8];
+        for (int h = 0; h < VB / UT; ++h) {
+          const C* p = bp + k * LS + at(UT * (t + UT * h));
+          C x[UT];
 #pragma unroll
-          for (int j = 0; j < 8; ++j) x[j] = p[j];
-          Dft<T, 8, false, true>::run(x);   // Z_m, m = t + 8 h + VB q; rows R m + k, and R (L - 1 - m) + R - k negated
+          for (int j = 0; j < UT; ++j) x[j] = p[j];
+          Dft<T, UT, false, true>::run(x);   // Z_m, m = t + UT h + VB q; rows R m + k, and R (L - 1 - m) + R - k negated
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            z[h + VB / 8 * q] = x[q];
-            z[HV + HV - 1 - (h + VB / 8 * q)] = x[4 + q];
+          for (int q = 0; q < UT / 2; ++q) {
+            z[h + VB / UT * q] = x[q];
+            z[HV + HV - 1 - (h + VB / UT * q)] = x[UT / 2 + q];
           }
         }
       }
@@ -379,7 +382,7 @@ template <class T, int N> struct Fold {
 #pragma unroll
       for (int j = 0; j < L; ++j) p[j + j / G] = z[j];
     } else {
-      const int k = s >> 3, t = s & 7;
+      const int k = s / UT, t = s % UT;
       if (k == 0) {
         fold_bt<T, VB>(z, t == 0);
         C* p = bp + at(VB * t);
@@ -387,36 +390,36 @@ template <class T, int N> struct Fold {
         for (int j = 0; j < VB; ++j) p[j + j / G] = z[j];
       } else {
 #pragma unroll
-        for (int h = 0; h < VB / 8; ++h) {
-          C x[8];
+        for (int h = 0; h < VB / UT; ++h) {
+          C x[UT];
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            x[q] = z[h + VB / 8 * q];
-            x[4 + q] = z[HV + HV - 1 - (h + VB / 8 * q)];
+          for (int q = 0; q < UT / 2; ++q) {
+            x[q] = z[h + VB / UT * q];
+            x[UT / 2 + q] = z[HV + HV - 1 - (h + VB / UT * q)];
           }
-          Dft<T, 8, true, false>::run(x);
-          C* p = bp + k * LS + at(8 * (t + 8 * h));
+          Dft<T, UT, true, false>::run(x);
+          C* p = bp + k * LS + at(UT * (t + UT * h));
 #pragma unroll
-          for (int j = 0; j < 8; ++j) p[j] = x[j];
+          for (int j = 0; j < UT; ++j) p[j] = x[j];
         }
       }
     }
   }
   static __device__ __forceinline__ void bt_mid(C* __restrict__ bp, int s, const C* __restrict__ tw) {
     if constexpr (BIG) {
-      const int k = s >> 3, t = s & 7;
+      const int k = s / UT, t = s % UT;
       if (k == 0) {
         if (t < UI) {
-          C va[8], vb[8];
+          C va[UT], vb[UT];
           const int part = t == 0 ? VB / 2 : VB - t;
 #pragma unroll
-          for (int r = 0; r < 8; ++r) {
+          for (int r = 0; r < UT; ++r) {
             va[r] = bp[at(VB * r + t)];
             vb[r] = bp[at(VB * r + part)];
           }
-          fold_at<T, 16, true, UI>(va, vb, t, tw + TW_A + TW_B);
+          fold_at<T, 2 * UT, true, UI>(va, vb, t, tw + TW_A + TW_B);
 #pragma unroll
-          for (int r = 0; r < 8; ++r) {
+          for (int r = 0; r < UT; ++r) {
             bp[at(VB * r + t)] = va[r];
             bp[at(VB * r + part)] = vb[r];
           }
@@ -426,10 +429,10 @@ template <class T, int N> struct Fold {
         const C* w = tw + TW_A + t;
         C x[VB];
 #pragma unroll
-        for (int i = 0; i < VB; ++i) x[i] = i == 0 ? p[0] : cmul(w[8 * i], p[i * (8 + 8 / G)]);
+        for (int i = 0; i < VB; ++i) x[i] = i == 0 ? p[0] : cmul(w[UT * i], p[i * (UT + UT / G)]);
         Dft<T, VB>::run(x);
 #pragma unroll
-        for (int i = 0; i < VB; ++i) p[i * (8 + 8 / G)] = x[i];
+        for (int i = 0; i < VB; ++i) p[i * (UT + UT / G)] = x[i];
       }
     }
   }

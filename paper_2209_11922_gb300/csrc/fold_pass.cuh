@@ -1,7 +1,7 @@
 // fold_pass.cuh - the axis passes of plans and batches on the two-step transforms of fold_dst.cuh: the folded DST-I of
 // Dirichlet axes and the Hartley transform of periodic ones.
 //
-// A CTA owns P pencil pairs (P a power of two) of one axis; thread tid works for pair tid % P as thread tid / P of
+// A CTA owns P pencil pairs of one axis; thread tid works for pair tid % P as thread tid / P of
 // it. What bounds these passes is the chain load - A - exchange - B - store and, at 3D sizes, HBM; so data
 // stays in registers wherever the next step starts from what the thread holds:
 //   strided axes (y, z; pair = two adjacent x columns): step A reads its rows straight from global memory
@@ -22,15 +22,15 @@ namespace etd {
 
 // Register budgets: FP32 plans with at most 16 values per thread take 3 CTAs of 256 threads per SM, those with up
 // to 32 two (128 registers); FP64 plans run CTAs of at most 128 threads, up to 16 values 3 per SM and 32 values 2,
-// and from N = 768 CTAs of 256 threads with the full register file.
+// and from N = 768 CTAs of 256 threads with the full register file; N = 2048 CTAs of 512 (FP64 256) threads.
 // The stage kernels with weight tables (TAB: 2D plans, whose few tiles give an SM one or two CTAs) take one fewer.
 // PER: periodic axes (FoldH), else Dirichlet (Fold).
 template <class T, int N, bool PER> using FoldOf = typename std::conditional<PER, FoldH<T, N>, Fold<T, N>>::type;
 template <class T, int N, bool PER, bool TAB = false> struct FoldBudget {
   using F = FoldOf<T, N, PER>;
-  static constexpr int VALS = F::R > F::VB ? F::R : F::VB;
-  static constexpr int THREADS = sizeof(T) == 4 || F::L == 128 ? 256 : 128;
-  static constexpr int BLOCKS = sizeof(T) == 8 && F::L == 128 ? 1 : (VALS <= 16 ? 3 : 2) - (TAB ? 1 : 0);
+  static constexpr int VALS = F::L == 256 ? 32 : (F::R > F::VB ? F::R : F::VB);   // (L = 256: unit 0's inner radix)
+  static constexpr int THREADS = F::L == 256 && sizeof(T) == 4 ? 512 : sizeof(T) == 4 || F::L >= 128 ? 256 : 128;
+  static constexpr int BLOCKS = F::L == 256 || (sizeof(T) == 8 && F::L == 128) ? 1 : (VALS <= 16 ? 3 : 2) - (TAB ? 1 : 0);
 };
 
 // Operations of a fold kernel: PassOp, and the transform along x.
@@ -106,8 +106,14 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
   static_assert(F::UA == TPP, "one A unit per thread");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int tid = threadIdx.x, NT = blockDim.x, P = A.P, LP = A.lp;
-  const int lg = 31 - __clz(P);
-  const int p = tid & (P - 1), l = tid >> lg;
+  int p, l;
+  if (P & (P - 1)) {   // 12, 6 or 3 pairs: x extents that are odd multiples of 8 or less
+    l = tid / P;
+    p = tid - l * P;
+  } else {
+    p = tid & (P - 1);
+    l = tid >> (31 - __clz(P));
+  }
   C* tw = reinterpret_cast<C*>(smem_raw);
   C* buf = tw + F::TWN;
   C* const bp = buf + p * LP;
@@ -320,10 +326,10 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
   F::a(va, vb, l, tw);
   F::a_put(bp, l, va, vb);
   __syncthreads();
-  // exchange inside the units of step B: the 8 threads of a unit are one warp up to P = 4
+  // exchange inside the units of step B: the threads of a unit lie in one warp where P divides a warp's share of them
   auto unit_sync = [&]() {
     if constexpr (F::BIG) {
-      if (P <= 4) __syncwarp();
+      if (P * F::UT <= 32 && (P & (P - 1)) == 0) __syncwarp();
       else __syncthreads();
     }
   };
@@ -438,7 +444,7 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
         if constexpr (PER) {
           if (A.flog != T(0)) {
             const T fg = A.flog;
-#pragma unroll 2
+#pragma unroll 4
             for (int i = 0; i < VB; ++i) {   // a loop: artanh's code once
               const C w = bp[F::own_off(s, i)];
               bp[F::own_off(s, i)] = C{fg * artanh_(w.x), fg * artanh_(w.y)};
