@@ -27,6 +27,7 @@ LENGTHS = [4, 8, 16, 32, 64, 128, 256, 512, 1024, 2048, 6, 12, 24, 48, 96, 192, 
 FOLD = [32, 48, 64, 96, 128, 192, 256, 384, 512, 768, 1024, 1536, 2048]   # fold_has() of fold_dst.cuh
 # foldh_has() of fold_dst.cuh
 FOLDH = {"f32": [32, 48, 64, 96, 128, 192, 256, 384, 512], "f64": []}
+FOLDM = {"f32": [192, 256, 384, 512], "f64": []}   # foldm_has()
 TYPES = {"f32": "float", "f64": "double"}
 
 
@@ -54,24 +55,24 @@ def generate() -> list:
     srcs = []
     decls, rows = [], []
     for tk, tn in TYPES.items():
-        # transform variants (enum Variant of dst_engine.cuh): the two-step kernels (Dirichlet axes 3, periodic axes 4),
+        # transform variants (enum Variant of dst_engine.cuh): the two-step kernels (Dirichlet axes 3 and 6, periodic axes 4),
         # and for lengths without a two-step plan 2 Hartley, 1 odd extension (FP32 only; 1024 for the split-radix route's
         # plans) and 0 half-length recurrence (FP64 64, 1536 and 2048 too, for
         # few pencils)
-        for v, per, lengths in (("fold", "false", FOLD), ("foldh", "true", FOLDH[tk])):
+        for v, kind, lengths in (("fold", "V_FOLD", FOLD), ("foldm", "V_FOLDM", FOLDM[tk]), ("foldh", "V_FOLDH", FOLDH[tk])):
             for n in lengths:
                 name = f"kinfo_{tk}_{v}_{n}"
                 path = os.path.join(GEN, f"inst_{tk}_{v}_{n}.cu")
                 _write_if_changed(path, (
                     '#include "fold_pass.cuh"\n'
                     "namespace etd {\n"
-                    f"KernelInfo {name}() {{ return fold_info<{tn}, {n}, {per}>(); }}\n"
+                    f"KernelInfo {name}() {{ return fold_info<{tn}, {n}, {kind}>(); }}\n"
                     "}  // namespace etd\n"))
                 srcs.append(path)
                 decls.append(f"KernelInfo {name}();")
                 rows.append(f"    {name}(),")
         for v, o in ((("odd", 1), ("rec", 0), ("hart", 2)) if tk == "f32" else (("rec", 0), ("hart", 2))):
-            for n in [m for m in LENGTHS if m not in ([m for m in FOLDH[tk] if m != 512] if v == "hart" else FOLD)] + {"odd": [1024], "rec": [64, 1536, 2048] * (tk == "f64")}.get(v, []):
+            for n in [m for m in LENGTHS if m not in ([] if v == "hart" else FOLD)] + {"odd": [1024], "rec": [64, 1536, 2048] * (tk == "f64")}.get(v, []):
                 name = f"kinfo_{tk}_{v}_{n}"
                 path = os.path.join(GEN, f"inst_{tk}_{v}_{n}.cu")
                 _write_if_changed(path, (

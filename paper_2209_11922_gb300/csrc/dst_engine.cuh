@@ -217,10 +217,10 @@ __device__ __forceinline__ void Dft<T, R, NI, NO>::run(Cx<T>* x) {
 template <int... Rs> struct Radices {};
 template <class T, int N, bool ODD> struct FftPlan;
 // Transform variant of a kernel (template argument VAR): the two DST-I forms and the Hartley form.
-// The Hartley variant runs the recurrence variant's length-N FFT plan; V_FOLD names the folded odd extension
+// The Hartley variant runs the recurrence variant's length-N FFT plan; V_FOLD and V_FOLDM name the folded odd extension
 // and V_FOLDH the two-step Hartley form of fold_dst.cuh, V_DENSE the dense products of dense_pass.cuh, which have kernels
 // of their own.
-enum Variant : int { V_REC = 0, V_ODD = 1, V_HART = 2, V_FOLD = 3, V_FOLDH = 4, V_DENSE = 5 };
+enum Variant : int { V_REC = 0, V_ODD = 1, V_HART = 2, V_FOLD = 3, V_FOLDH = 4, V_DENSE = 5, V_FOLDM = 6 };
 #define ETD_PLAN(TYPE, NN, ODD_, TPP_, ...)                \
   template <> struct FftPlan<TYPE, NN, ODD_> {             \
     static constexpr bool ODD = ODD_;                      \

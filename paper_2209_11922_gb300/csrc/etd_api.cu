@@ -110,20 +110,25 @@ int env_int(const char* name, int dflt) {
 // per transform where an FFT pass costs its longest thread, 16 to 60 thousand cycles at these lengths. The lines lie
 // where the two were equal (us per ETDRK2 step, dense against FFT: 64^2 19.5 / 138, 128^2 35 / 157, 256^2 148 / 173,
 // 48^3 108 / 251; 64^3 259 / 232 by the recurrence, 96^3 ETDRK1 490 / 271).
-int dst_variant(const etd_options& o, int64_t n, int64_t pairs, bool batch) {
+int dst_variant(const etd_options& o, int axis, int64_t n, int64_t pairs, bool batch) {
   if (o.dtype == ETD_F64 && !batch) {
     if (n <= 256 && 2 * pairs * n * n <= (n == 64 ? 12000000 : 20000000)) return V_DENSE;
     // N = 64 up to 4000 pairs, where the folded plan's 4 threads per pair leave schedulers idle, and N = 1536 and 2048
     // over few pencils: the recurrence's threads hold half the values (8, and 16 against 24 and 32; 64^3 286 us by the
     // folded plan, 2048 x 64 222 against 307)
-    if (o.bc == ETD_BC_DIRICHLET && ((n == 64 && pairs <= 4000) || ((n == 1536 || n == 2048) && pairs <= 128))) return V_REC;
+    if (o.bc == ETD_BC_DIRICHLET && ((n == 64 && pairs <= 4000) || ((n == 1536 || n == 2048) && pairs <= 256))) return V_REC;
   }
+  // periodic x axes over few pencils whose two-step plan holds 24 or 32 values per thread: the general kernels' 12 to 16
+  // (256 x 24 x 64 255 us per 12 steps against 217, 384 x 192 125 against 111; N = 128 holds 16 and is faster)
+  if (o.bc == ETD_BC_PERIODIC && axis == 0 && !batch && (n == 96 || n >= 192) && pairs < 1100) return V_HART;
   if (o.bc == ETD_BC_PERIODIC) return foldh_has(o.dtype == ETD_F32 ? 4 : 8, (int)n, pairs) ? V_FOLDH : V_HART;
+  // few pencils: the plans with many threads (256^2 876 -> 636 us per 40 steps, 768 x 192 560 -> 476; N = 128 gains nothing)
+  if (o.dtype == ETD_F32 && !batch && foldm_has((int)n) && pairs <= 2000) return V_FOLDM;
   if (fold_has((int)n)) return V_FOLD;
   return o.dtype == ETD_F32 && o.route == ETD_ROUTE_FFT ? V_ODD : V_REC;
 }
 
-bool two_step(const KernelInfo& k) { return k.odd == V_FOLD || k.odd == V_FOLDH; }
+bool two_step(const KernelInfo& k) { return k.odd == V_FOLD || k.odd == V_FOLDM || k.odd == V_FOLDH; }
 
 bool supported_length(int64_t n) {
   if (n < 4 || n > 2048) return false;
@@ -275,36 +280,34 @@ etd_status make_split_launch(etd_plan_s* pl, int op, int axis, const void* in0, 
   return ETD_OK;
 }
 
-// Dense user field <-> pitched field (PACK / UNPACK): four rows per round and block, their loads in flight together.
+// Dense user field <-> pitched field (PACK / UNPACK): groups of rows of about 1024 elements per block, a thread's
+// elements 256 apart, their loads in flight together.
+constexpr int kPackElems = 1024;
 template <class T>
 __global__ void __launch_bounds__(256) pack_kernel(const PassArgs<T> A) {
   griddep_wait();
   constexpr int U = 4;
   const int cut = A.user_slot;   // 1: Dirichlet (index 0 is the boundary), 0: periodic
-  const int rows = A.ny * A.nz;
-  for (int r0 = blockIdx.x; r0 < rows; r0 += U * gridDim.x) {
-    long long d[U];   // dense start of the row, -1: boundary row or past the end
+  const int rows = A.ny * A.nz, rpb = A.P, n = rpb * A.nx;   // rows per block
+  const int r0 = blockIdx.x * rpb;
+  for (int i0 = threadIdx.x; i0 < n; i0 += U * 256) {
+    T v[U];
+    long long d[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int r = r0 + u * gridDim.x, z = r / A.ny, y = r - z * A.ny;
-      const bool in = r < rows && y >= cut && (A.ndim == 2 || z >= cut);
-      d[u] = in ? ((long long)(A.ndim == 3 ? z - cut : 0) * (A.ny - cut) + (y - cut)) * (A.nx - cut) - cut : -2;
+      const int i = i0 + u * 256, rr = i / A.nx, x = i - rr * A.nx, r = r0 + rr, z = r / A.ny, y = r - z * A.ny;
+      const bool in = i < n && r < rows && x >= cut && y >= cut && (A.ndim == 2 || z >= cut);
+      d[u] = in ? ((long long)(A.ndim == 3 ? z - cut : 0) * (A.ny - cut) + (y - cut)) * (A.nx - cut) + (x - cut) : -1;
+      v[u] = T(0);
+      if (in) v[u] = A.op == OP_PACK ? A.in0[d[u]] : A.in0[(size_t)r0 * A.nx + i];
     }
-    for (int x = threadIdx.x; x < A.nx; x += blockDim.x) {
-      T v[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const bool in = d[u] > -2 && x >= cut;
-        v[u] = T(0);
-        if (in) v[u] = A.op == OP_PACK ? A.in0[d[u] + x] : A.in0[(size_t)(r0 + u * gridDim.x) * A.nx + x];
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        if (A.op == OP_PACK) {
-          if (r0 + u * (int)gridDim.x < rows) A.out0[(size_t)(r0 + u * gridDim.x) * A.nx + x] = v[u];
-        } else if (d[u] > -2 && x >= cut) {
-          A.out0[d[u] + x] = v[u];
-        }
+    for (int u = 0; u < U; ++u) {
+      const int i = i0 + u * 256;
+      if (A.op == OP_PACK) {
+        if (i < n && r0 + i / A.nx < rows) A.out0[(size_t)r0 * A.nx + i] = v[u];
+      } else if (d[u] >= 0) {
+        A.out0[d[u]] = v[u];
       }
     }
   }
@@ -342,7 +345,8 @@ etd_status make_fold_launch(etd_plan_s* pl, const KernelInfo* k, PassArgs<T>& a,
         pick = q;
       }
     }
-    if (a.axis == 0 || pick > pmin) pmin = pick;
+    // (N = 2048: two pairs, whose units exchange within a warp, while the CTAs are few)
+    if (a.axis == 0 || pick > pmin || (k->radix[1] == 256 && pairs / 4 < sms)) pmin = pick;
   }
   if (a.axis == 0) {
     while (P > pmin && pairs / P < 2 * sms) P /= 2;
@@ -443,9 +447,9 @@ etd_status make_launch(etd_plan_s* pl, int op, int axis, const void* in0, const 
     a.in0 = static_cast<const T*>(in0);
     a.out0 = static_cast<T*>(out0);
     a.user_slot = pl->periodic ? 0 : 1;
-    const long long blocks = ((long long)pl->ny * pl->nz + 3) / 4;   // four rows each
+    a.P = pl->nx < kPackElems ? kPackElems / pl->nx : 1;
     L.fn = reinterpret_cast<const void*>(&pack_kernel<T>);
-    L.grid = dim3((unsigned)(blocks < 16LL * pl->num_sms ? blocks : 16LL * pl->num_sms));
+    L.grid = dim3((unsigned)(((long long)pl->ny * pl->nz + a.P - 1) / a.P));
     L.block = dim3(256);
     L.smem = 0;
     L.kind = kind;
@@ -578,11 +582,11 @@ etd_status launch(const Launch& L, cudaStream_t s) {
 
 // Which launches of a time step take programmatic dependent launch. It hides a launch's latency (2 to 4 us of a step),
 // but CTAs that start while their predecessor drains go to the SMs it leaves free, several to one SM, and stay there:
-// where the grid is a few large CTAs per SM the pass then takes as long as the SM with the most (1023^2 FP64 ETDRK1,
-// 128 CTAs: 298 us per step against 216; FP32 ETDRK2 31.9 against 28.7). So a launch goes without when it and its
-// predecessor do not fit on distinct SMs, its CTAs are large enough to load an SM (256 threads; FP64, whose units a
-// warp keeps for 64 cycles, 48: 24 x 256 x 64 ETDRK1 293 us per step against 183), more of them fit on an SM than an even spread puts there, and there are too few of them
-// for the imbalance to average out.
+// where a pass is bound by the warps of the busiest SM it then takes as long as that one. So a launch goes without when
+// it and its predecessor do not fit on distinct SMs, more of its CTAs fit on an SM than an even spread puts there, and
+// an SM's share loads it: FP64, whose units a warp keeps for 64 cycles, from four warps per SM on (24 x 256 x 64 ETDRK1
+// 259 us per step with, 149 without; 128 x 192 x 24 599 and 369; 1023^2 298 and 216; many waves lose 0.4%); FP32 CTAs of
+// 256 threads that would be one per SM, on at least a third of the SMs (1023^2 ETDRK2 31.9 and 28.7).
 void choose_pdl(std::vector<Launch>& step, int num_sms, int elem) {
   for (size_t i = 0; i < step.size(); ++i) {
     Launch& L = step[i];
@@ -593,8 +597,8 @@ void choose_pdl(std::vector<Launch>& step, int num_sms, int elem) {
       cudaGetLastError();
       continue;
     }
-    L.pdl = !(grid + prev > num_sms && grid < 4LL * num_sms && threads >= (elem == 8 ? 48 : 256) &&
-              occ > (grid + num_sms - 1) / num_sms);
+    const bool loads = elem == 8 ? grid * ((threads + 31) / 32) >= 4LL * num_sms : threads >= 256 && grid <= num_sms && 3 * grid >= num_sms;
+    L.pdl = !(grid + prev > num_sms && occ > (grid + num_sms - 1) / num_sms && loads);
   }
 }
 
@@ -1935,7 +1939,7 @@ etd_status etd_plan_create(etd_plan* out, int ndim, const int64_t* N, const doub
   pl->opt = o;
   pl->elem = (o.dtype == ETD_F32) ? 4 : 8;
   for (int a = 0; a < ndim; ++a) {
-    pl->odd[a] = dst_variant(o, N[a], N[0] * N[1] * (ndim == 3 ? N[2] : 1) / N[a] / 2, false);
+    pl->odd[a] = dst_variant(o, a, N[a], N[0] * N[1] * (ndim == 3 ? N[2] : 1) / N[a] / 2, false);
   }
   // ETD_ROUTE_FFT_SPLIT: FP32 Dirichlet axes of length 1024 take the split-radix kernels (the strided
   // passes need an x extent that is a multiple of 4); every other axis the AUTO choice.
@@ -1970,7 +1974,9 @@ etd_status etd_plan_create(etd_plan* out, int ndim, const int64_t* N, const doub
   if (st != ETD_OK) return bail(st);
   // per-mode phi-function weights of the y passes of 2D plans on the FFT routes (at most 64 MiB)
   const size_t coef_bytes = pl->nfield * (pl->scheme == 2 ? 3 : 1) * (size_t)pl->elem;
-  if (ndim == 2 && !gemm && coef_bytes <= ((size_t)64 << 20)) {
+  // (FP32 on the general Hartley kernels evaluates them: staging the tables costs those a CTA per SM, 2048 x 1024
+  // periodic 81.5 us per step against 74.9)
+  if (ndim == 2 && !gemm && coef_bytes <= ((size_t)64 << 20) && !(pl->elem == 4 && pl->odd[1] == V_HART)) {
     st = pl->elem == 4 ? upload_coef_tables<float>(pl) : upload_coef_tables<double>(pl);
     if (st != ETD_OK) return bail(st);
   }
@@ -2346,8 +2352,8 @@ etd_status etd_batch_create(etd_batch* out, int count, const int64_t* N, const d
     b->hx.push_back(h[2 * i]);
     b->hy.push_back(h[2 * i + 1]);
     b->Dv.push_back(D[i]);
-    b->oddx.push_back(dst_variant(o, N[2 * i], 1024, true));   // the group's pairs of all problems fill the GPU
-    b->oddy.push_back(dst_variant(o, N[2 * i + 1], 1024, true));
+    b->oddx.push_back(dst_variant(o, 0, N[2 * i], 1024, true));   // the group's pairs of all problems fill the GPU
+    b->oddy.push_back(dst_variant(o, 1, N[2 * i + 1], 1024, true));
   }
   if (cudaGetDevice(&b->device) != cudaSuccess) {
     delete b;

@@ -37,9 +37,9 @@ namespace etd {
 // L <= 32: step B is one register DFT per unit. L = 64, 128: units of UT = 8 threads, L/8 values each (L/8 x 8);
 // L = 256: units of 16 threads (16 x 16).
 // G: one padding slot every G positions (G divides L, so slot offsets are compile-time constants).
-template <class T, int N> struct FoldPlan { static constexpr int R = 0, L = 0, TPP = 1, G = 1; };
+template <class T, int N, bool MANY = false> struct FoldPlan { static constexpr int R = 0, L = 0, TPP = 1, G = 1; };
 #define ETD_FOLD(NN, R_, L_, TPP_, G_)                                             \
-  template <class T> struct FoldPlan<T, NN> {                                      \
+  template <class T> struct FoldPlan<T, NN, false> {                               \
     static_assert(R_ * L_ == 2 * NN, "R L = 2N");                                  \
     static constexpr int R = R_, L = L_, TPP = TPP_, G = G_;                       \
   };
@@ -62,10 +62,21 @@ ETD_FOLD(2048, 16, 256, 128, 16)
 // (L = 64: eight values) than FP32 (256^2 ETDRK2 326 -> 158 us per step against R = 32, L = 16). Shorter axes keep
 // the plans that leave no lane idle in step B (64^3: 233 us; R = 8, L = 16 idles half of them there, 350 us).
 #define ETD_FOLD64(NN, R_, L_, TPP_, G_)                                           \
-  template <> struct FoldPlan<double, NN> {                                        \
+  template <> struct FoldPlan<double, NN, false> {                                 \
     static_assert(R_ * L_ == 2 * NN, "R L = 2N");                                  \
     static constexpr int R = R_, L = L_, TPP = TPP_, G = G_;                       \
   };
+// MANY: FP32 plans over few pencils, the same many-threads form (an FP32 pass over few pencils costs its longest chain).
+#define ETD_FOLDM(NN, R_, L_, TPP_, G_)                                            \
+  template <> struct FoldPlan<float, NN, true> {                                   \
+    static_assert(R_ * L_ == 2 * NN, "R L = 2N");                                  \
+    static constexpr int R = R_, L = L_, TPP = TPP_, G = G_;                       \
+  };
+ETD_FOLDM(192, 6, 64, 32, 8)
+ETD_FOLDM(256, 8, 64, 32, 8)
+ETD_FOLDM(384, 12, 64, 32, 8)
+ETD_FOLDM(512, 16, 64, 32, 8)
+#undef ETD_FOLDM
 ETD_FOLD64(192, 6, 64, 32, 8)
 ETD_FOLD64(256, 8, 64, 32, 8)
 ETD_FOLD64(384, 12, 64, 32, 8)
@@ -73,6 +84,7 @@ ETD_FOLD64(512, 16, 64, 32, 8)
 ETD_FOLD64(2048, 32, 128, 64, 8)   // R = 16, L = 256 on 128 threads: 2048 x 1024 ETDRK2 1016 us per step against 891
 #undef ETD_FOLD64
 
+constexpr bool foldm_has(int n) { return n == 192 || n == 256 || n == 384 || n == 512; }   // FP32
 constexpr bool fold_has(int n) {
   return n == 32 || n == 48 || n == 64 || n == 96 || n == 128 || n == 192 || n == 256 || n == 384 || n == 512 ||
          n == 768 || n == 1024 || n == 1536 || n == 2048;
@@ -237,8 +249,8 @@ __device__ __forceinline__ void fold_bt(Cx<T> (&z)[L], bool special) {
 }
 
 // Geometry and the two steps of one axis transform for a thread (pair buffer bp, thread l of the pair).
-template <class T, int N> struct Fold {
-  using Plan = FoldPlan<T, N>;
+template <class T, int N, bool MANY = false> struct Fold {
+  using Plan = FoldPlan<T, N, MANY>;
   using C = Cx<T>;
   static constexpr int R = Plan::R, L = Plan::L, TPP = Plan::TPP, G = Plan::G;
   static constexpr int H = R / 2;                       // units of step B

@@ -24,10 +24,11 @@ namespace etd {
 // to 32 two (128 registers); FP64 plans run CTAs of at most 128 threads, up to 16 values 3 per SM and 32 values 2,
 // and from N = 768 CTAs of 256 threads with the full register file; N = 2048 CTAs of 512 (FP64 256) threads.
 // The stage kernels with weight tables (TAB: 2D plans, whose few tiles give an SM one or two CTAs) take one fewer.
-// PER: periodic axes (FoldH), else Dirichlet (Fold).
-template <class T, int N, bool PER> using FoldOf = typename std::conditional<PER, FoldH<T, N>, Fold<T, N>>::type;
-template <class T, int N, bool PER, bool TAB = false> struct FoldBudget {
-  using F = FoldOf<T, N, PER>;
+// KIND: V_FOLD, V_FOLDM (Dirichlet) or V_FOLDH (periodic).
+template <class T, int N, int KIND>
+using FoldOf = typename std::conditional<KIND == V_FOLDH, FoldH<T, N>, Fold<T, N, KIND == V_FOLDM>>::type;
+template <class T, int N, int KIND, bool TAB = false> struct FoldBudget {
+  using F = FoldOf<T, N, KIND>;
   static constexpr int VALS = F::L == 256 ? 32 : (F::R > F::VB ? F::R : F::VB);   // (L = 256: unit 0's inner radix)
   static constexpr int THREADS = F::L == 256 && sizeof(T) == 4 ? 512 : sizeof(T) == 4 || F::L >= 128 ? 256 : 128;
   static constexpr int BLOCKS = F::L == 256 || (sizeof(T) == 8 && F::L == 128) ? 1 : (VALS <= 16 ? 3 : 2) - (TAB ? 1 : 0);
@@ -93,11 +94,38 @@ template <class T> __device__ __forceinline__ Cx<T> phi2_pair(Cx<T> zeta, Cx<T> 
   return p2;
 }
 
+// artanh of two values. FP32: artanh x = (k/2) ln 2 + artanh s with s = (a - 2^k b)/(a + 2^k b), a = 1 + x, b = 1 - x and
+// 2^k next to a/b, so that |s| <= 1/5 and the odd series up to s^11 suffices; s = x where k = 0. Component-wise packed;
+// over (-1, 1) its relative error is 5.0e-8 rms and 3.6e-7 (3 ulp, the documented bound of atanhf) at most. Not finite for
+// |x| >= 1.
+__device__ __forceinline__ Cx<double> artanh2(Cx<double> x) { return Cx<double>{atanh(x.x), atanh(x.y)}; }
+__device__ __forceinline__ Cx<float> artanh2(Cx<float> x) {
+  const Cx<float> one{1.f, 1.f}, a = one + x, b = one - x;
+  // k from the exponent of a / b against 3/4 (the quotient's approximation moves the line by an ulp, which the series
+  // absorbs); |x| >= 1 gives a NaN below
+  const float qx = a.x * rcp_approx(b.x), qy = a.y * rcp_approx(b.y);
+  const int kx = (__float_as_int(qx) - 0x3f400000) >> 23, ky = (__float_as_int(qy) - 0x3f400000) >> 23;
+  const Cx<float> K{__int_as_float((kx + 127) << 23), __int_as_float((ky + 127) << 23)};
+  const Cx<float> kb = mul2(K, b), num = a - kb, den = a + kb;   // K b is exact
+  const Cx<float> q = mul2(num, rcp2(den));
+  const Cx<float> s{kx == 0 ? x.x : q.x, ky == 0 ? x.y : q.y}, s2 = mul2(s, s);
+  Cx<float> p{1.f / 11, 1.f / 11};
+  p = fma2(p, s2, Cx<float>{1.f / 9, 1.f / 9});
+  p = fma2(p, s2, Cx<float>{1.f / 7, 1.f / 7});
+  p = fma2(p, s2, Cx<float>{1.f / 5, 1.f / 5});
+  p = fma2(p, s2, Cx<float>{1.f / 3, 1.f / 3});
+  const Cx<float> t = fma2(mul2(s, s2), p, s);
+  const Cx<float> r = fma2(Cx<float>{(float)kx, (float)ky}, Cx<float>{0.34657359027997264f, 0.34657359027997264f}, t);
+  const float nan = __int_as_float(0x7fffffff);
+  return Cx<float>{fabsf(x.x) < 1.f ? r.x : nan, fabsf(x.y) < 1.f ? r.y : nan};
+}
+
 // TAB: the stage weights come from the plan's per-mode tables (2D plans), else from phi evaluated per mode.
 // dense: the caller's field (ENTRY source, EXIT destination).
-template <class T, int N, bool PER, int OP, bool TAB>
+template <class T, int N, int KIND, int OP, bool TAB>
 __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, T* dense) {
-  using F = FoldOf<T, N, PER>;
+  using F = FoldOf<T, N, KIND>;
+  constexpr bool PER = KIND == V_FOLDH;
   using C = Cx<T>;
   using VT = typename V2<T>::type;
   constexpr int H = F::H, QB = F::QB, VB = F::VB, HV = F::HV, TPP = F::TPP;
@@ -195,7 +223,7 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
   if (A.step_inc && blockIdx.x == 0 && tid == 0) atomicAdd(A.step_inc, 1ULL);
 
   // ---- x axis: staged rows
-  constexpr int V = sizeof(T) == 4 ? 4 : 2;                 // elements per vector access
+  constexpr int V = sizeof(T) == 4 && (N / 4) % TPP == 0 ? 4 : 2;   // elements per vector access
   using VL = typename std::conditional<V == 4, float4, VT>::type;
   constexpr int RV = N / V;                                  // vectors per row
   constexpr int CNT = RV / TPP;                              // per thread and row
@@ -263,28 +291,32 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
       reinterpret_cast<VL*>(dst + (size_t)rb * A.nx)[k] = vb;
     }
   };
-  // dense user rows: nx - 1 interior values of the rows with y >= 1 (and z >= 1); periodic: the pitched rows
+  // index 0 of a row in the dense user field: nx - 1 interior values of the rows with y >= 1 (and z >= 1); periodic: the
+  // pitched rows
   auto dense_row = [&](int r) -> long long {
     if constexpr (PER) return (long long)r * A.nx;
     const int y = r % A.ny, z = r / A.ny;
-    if (y == 0 || (A.ndim == 3 && z == 0)) return -1;
-    return ((A.ndim == 3 ? (long long)(z - 1) * (A.ny - 1) : 0LL) + (y - 1)) * (A.nx - 1);
+    if (y == 0 || (A.ndim == 3 && z == 0)) return -2;
+    return ((A.ndim == 3 ? (long long)(z - 1) * (A.ny - 1) : 0LL) + (y - 1)) * (A.nx - 1) - 1;
   };
+  long long* drow = reinterpret_cast<long long*>(own);   // ENTRY, EXIT: [2 P]
 
-  constexpr int X0 = PER ? 0 : 1;   // dense column of pitched index x is x - X0
+  constexpr int X0 = PER ? 0 : 1;   // first index with a value
   C va[H], vb[H];
   const size_t ostep = (size_t)F::STEP * rs * sizeof(T);   // bytes between a thread's consecutive rows after step B
   if constexpr (XAX) {
     if constexpr (OP == OP_ENTRY) {
-#pragma unroll 4
-      for (int pp = 0; pp < P; ++pp) {
-        const long long da = q0 + pp < A.npairs ? dense_row(2 * (q0 + pp)) : -1, db = q0 + pp < A.npairs ? dense_row(2 * (q0 + pp) + 1) : -1;
-        for (int x = tid; x < N; x += NT) {
-          C c{T(0), T(0)};
-          if (x >= X0 && da >= 0) c.x = dense[da + x - X0];
-          if (x >= X0 && db >= 0) c.y = dense[db + x - X0];
-          buf[pp * LP + F::at(x)] = c;
-        }
+      // dense starts of the tile's rows (index 0), -2 for boundary rows and rows past the end, once per row
+      for (int i = tid; i < 2 * P; i += NT) drow[i] = q0 + (i >> 1) < A.npairs ? dense_row(2 * q0 + i) : -2;
+      __syncthreads();
+#pragma unroll 8
+      for (int i = tid; i < P * N; i += NT) {
+        const int pp = i / N, x = i - pp * N;
+        const long long da = drow[2 * pp], db = drow[2 * pp + 1];
+        C c{T(0), T(0)};
+        if (x >= X0 && da > -2) c.x = dense[da + x];
+        if (x >= X0 && db > -2) c.y = dense[db + x];
+        buf[pp * LP + F::at(x)] = c;
       }
     } else {
       stage_in(A.in0);
@@ -374,15 +406,15 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
     __syncthreads();
     griddep_launch_dependents();
     if constexpr (OP == OP_EXIT) {
-#pragma unroll 4
-      for (int pp = 0; pp < P; ++pp) {
-        if (q0 + pp >= A.npairs) continue;
-        const long long da = dense_row(2 * (q0 + pp)), db = dense_row(2 * (q0 + pp) + 1);
-        for (int x = tid; x < N; x += NT) {
-          const C c = buf[pp * LP + F::at(x)];
-          if (x >= X0 && da >= 0) dense[da + x - X0] = c.x;
-          if (x >= X0 && db >= 0) dense[db + x - X0] = c.y;
-        }
+      for (int i = tid; i < 2 * P; i += NT) drow[i] = q0 + (i >> 1) < A.npairs ? dense_row(2 * q0 + i) : -2;
+      __syncthreads();
+#pragma unroll 8
+      for (int i = tid; i < P * N; i += NT) {
+        const int pp = i / N, x = i - pp * N;
+        const long long da = drow[2 * pp], db = drow[2 * pp + 1];
+        const C c = buf[pp * LP + F::at(x)];
+        if (x >= X0 && da > -2) dense[da + x] = c.x;
+        if (x >= X0 && db > -2) dense[db + x] = c.y;
       }
     } else {
       stage_out(A.out0);
@@ -446,8 +478,7 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
             const T fg = A.flog;
 #pragma unroll 4
             for (int i = 0; i < VB; ++i) {   // a loop: artanh's code once
-              const C w = bp[F::own_off(s, i)];
-              bp[F::own_off(s, i)] = C{fg * artanh_(w.x), fg * artanh_(w.y)};
+              bp[F::own_off(s, i)] = fg * artanh2(bp[F::own_off(s, i)]);
             }
 #pragma unroll
             for (int i = 0; i < VB; ++i) z[i] = z[i] + bp[F::own_off(s, i)];
@@ -572,22 +603,22 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
   }
 }
 
-template <class T, int N, bool PER, int OP, bool TAB>
-__global__ void __launch_bounds__(FoldBudget<T, N, PER>::THREADS, FoldBudget<T, N, PER, TAB>::BLOCKS)
+template <class T, int N, int KIND, int OP, bool TAB>
+__global__ void __launch_bounds__(FoldBudget<T, N, KIND>::THREADS, FoldBudget<T, N, KIND, TAB>::BLOCKS)
     fold_kernel(const PassArgs<T> A) {
-  fold_body<T, N, PER, OP, TAB>(A, (int)blockIdx.x, OP == OP_ENTRY ? const_cast<T*>(A.in0) : A.out0);
+  fold_body<T, N, KIND, OP, TAB>(A, (int)blockIdx.x, OP == OP_ENTRY ? const_cast<T*>(A.in0) : A.out0);
 }
 
 // Batches: CTA b works on tile map[b].y of problem descs[map[b].x]; entry and exit passes take the caller's field
 // from user[].
-template <class T, int N, bool PER, int OP>
-__global__ void __launch_bounds__(FoldBudget<T, N, PER>::THREADS, FoldBudget<T, N, PER>::BLOCKS)
+template <class T, int N, int KIND, int OP>
+__global__ void __launch_bounds__(FoldBudget<T, N, KIND>::THREADS, FoldBudget<T, N, KIND>::BLOCKS)
     fold_kernel_batched(const PassArgs<T>* __restrict__ descs, const int2* __restrict__ map, T* const* __restrict__ user) {
   const int2 m = map[blockIdx.x];
   const PassArgs<T>& A = descs[m.x];   // read in place
   T* dense = nullptr;
   if (OP == OP_ENTRY || OP == OP_EXIT) dense = user[A.user_slot];
-  fold_body<T, N, PER, OP, false>(A, m.y, dense);
+  fold_body<T, N, KIND, OP, false>(A, m.y, dense);
 }
 
 // Shared memory of a launch: op, pairs per CTA, pair stride, tables / staged weights.
@@ -595,32 +626,32 @@ inline size_t fold_smem_bytes(const KernelInfo& k, int op, int P, int lp, bool t
   const size_t c = 2 * (size_t)k.elem;
   size_t b = ((size_t)k.twn + (size_t)P * lp) * c;
   b = (b + 15) & ~(size_t)15;
-  if (!fold_is_stage(op)) return b;
+  if (!fold_is_stage(op)) return b + (op == OP_ENTRY || op == OP_EXIT ? 2 * (size_t)P * sizeof(long long) : 0);
   const size_t own = tab ? (size_t)k.own_vals * P * k.tpp : 0;
   b += own * c + (tab ? 2 : 5) * (size_t)k.N * k.elem;
   if (tab && staged) b += own * 2 * k.elem * (op == OP_S1S ? 2 : 1);
   return b;
 }
 
-template <class T, int N, bool PER> KernelInfo fold_info() {
-  using F = FoldOf<T, N, PER>;
+template <class T, int N, int KIND> KernelInfo fold_info() {
+  using F = FoldOf<T, N, KIND>;
   KernelInfo k{};
   k.N = N;
   k.tpp = F::TPP;
   k.lp = F::LP;
   k.elem = (int)sizeof(T);
-  k.fft_len = PER ? N : 2 * N;
-  k.odd = PER ? V_FOLDH : V_FOLD;
+  k.fft_len = KIND == V_FOLDH ? N : 2 * N;
+  k.odd = KIND;
   k.padg = F::G;
   k.twn = F::TWN;
   k.radix[0] = F::R;
   k.radix[1] = F::L;
-  k.min_blocks = FoldBudget<T, N, PER>::BLOCKS;
-  k.max_threads = FoldBudget<T, N, PER>::THREADS;
+  k.min_blocks = FoldBudget<T, N, KIND>::BLOCKS;
+  k.max_threads = FoldBudget<T, N, KIND>::THREADS;
   k.own_vals = F::QB * F::VB;
 #define ETD_FOLD_OP(OP)                                                                   \
-  k.fn_op[OP] = reinterpret_cast<const void*>(&fold_kernel<T, N, PER, OP, false>);             \
-  k.fn_batched_op[OP] = reinterpret_cast<const void*>(&fold_kernel_batched<T, N, PER, OP>);
+  k.fn_op[OP] = reinterpret_cast<const void*>(&fold_kernel<T, N, KIND, OP, false>);             \
+  k.fn_batched_op[OP] = reinterpret_cast<const void*>(&fold_kernel_batched<T, N, KIND, OP>);
   ETD_FOLD_OP(OP_ENTRY)
   ETD_FOLD_OP(OP_EXIT)
   ETD_FOLD_OP(OP_REACT)
@@ -629,10 +660,10 @@ template <class T, int N, bool PER> KernelInfo fold_info() {
   ETD_FOLD_OP(OP_S1S)
   ETD_FOLD_OP(OP_S2S)
 #undef ETD_FOLD_OP
-  k.fn_tab[OP_RK1S] = reinterpret_cast<const void*>(&fold_kernel<T, N, PER, OP_RK1S, true>);
-  k.fn_tab[OP_S1S] = reinterpret_cast<const void*>(&fold_kernel<T, N, PER, OP_S1S, true>);
-  k.fn_tab[OP_S2S] = reinterpret_cast<const void*>(&fold_kernel<T, N, PER, OP_S2S, true>);
-  k.fn_x = reinterpret_cast<const void*>(&fold_kernel<T, N, PER, OP_TRANSFORM_X, false>);
+  k.fn_tab[OP_RK1S] = reinterpret_cast<const void*>(&fold_kernel<T, N, KIND, OP_RK1S, true>);
+  k.fn_tab[OP_S1S] = reinterpret_cast<const void*>(&fold_kernel<T, N, KIND, OP_S1S, true>);
+  k.fn_tab[OP_S2S] = reinterpret_cast<const void*>(&fold_kernel<T, N, KIND, OP_S2S, true>);
+  k.fn_x = reinterpret_cast<const void*>(&fold_kernel<T, N, KIND, OP_TRANSFORM_X, false>);
   return k;
 }
 
