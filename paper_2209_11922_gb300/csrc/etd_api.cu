@@ -584,7 +584,8 @@ etd_status launch(const Launch& L, cudaStream_t s) {
 // but CTAs that start while their predecessor drains go to the SMs it leaves free, several to one SM, and stay there:
 // where a pass is bound by the warps of the busiest SM it then takes as long as that one. So a launch goes without when
 // it and its predecessor do not fit on distinct SMs, more of its CTAs fit on an SM than an even spread puts there, and
-// an SM's share loads it: FP64, whose units a warp keeps for 64 cycles, from four warps per SM on (24 x 256 x 64 ETDRK1
+// an SM's share loads it: FP64, whose units a warp keeps for 64 cycles, from two warps per SM on, unless
+// equal grids of three or more CTAs per SM follow each other (24 x 256 x 64 ETDRK1
 // 259 us per step with, 149 without; 128 x 192 x 24 599 and 369; 1023^2 298 and 216; many waves lose 0.4%); FP32 CTAs of
 // 256 threads that would be one per SM, on at least a third of the SMs (1023^2 ETDRK2 31.9 and 28.7).
 void choose_pdl(std::vector<Launch>& step, int num_sms, int elem) {
@@ -597,7 +598,8 @@ void choose_pdl(std::vector<Launch>& step, int num_sms, int elem) {
       cudaGetLastError();
       continue;
     }
-    const bool loads = elem == 8 ? grid * ((threads + 31) / 32) >= 4LL * num_sms : threads >= 256 && grid <= num_sms && 3 * grid >= num_sms;
+    const bool loads = elem == 8 ? grid * ((threads + 31) / 32) >= 2LL * num_sms && !(grid == prev && grid >= 3LL * num_sms)
+                                 : threads >= 256 && grid <= num_sms && 3 * grid >= num_sms;
     L.pdl = !(grid + prev > num_sms && occ > (grid + num_sms - 1) / num_sms && loads);
   }
 }
