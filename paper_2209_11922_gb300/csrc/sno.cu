@@ -14,6 +14,7 @@
 #include "../../include/etd.h"
 #include "../../include/etd_sno.h"
 #include "sno_kernels.cuh"
+#include "sno_grad.cuh"
 #include "sno_layer.cuh"
 #include "sno_mma.cuh"
 
@@ -414,7 +415,80 @@ etd_status chan_reduce(etd_sno_s* m, const float* X, const float* y, const float
   if ((long long)B * C * nblk > m->part_len) return sfail(ETD_ERR_UNSUPPORTED, "reduction scratch too small");
   chan_dot_kernel<<<dim3(nblk, B * C), 256, 0, s>>>(X, y, C, m->npix, m->part);
   SNO_CUDA(cudaGetLastError());
-  chan_combine_kernel<<<(C + 127) / 128, 128, 0, s>>>(m->part, nblk, w, B, C, m->G + off, stride, 0);
+  chan_combine_kernel<<<C, 128, 0, s>>>(m->part, nblk, w, B, C, m->G + off, stride);
+  SNO_CUDA(cudaGetLastError());
+  return ETD_OK;
+}
+
+// Gradient with the kernels of sno_grad.cuh (C = 16 or 32, M <= 24): the order of operations of sno_backward.
+template <int C, int KIND>
+etd_status launch_point(const etd_sno_s* m, const GradPointArgs& g, cudaStream_t s) {
+  const long long warps = (g.np + 63) / 64 * g.B;
+  grad_point_kernel<C, KIND><<<(int)std::min<long long>((warps + 7) / 8, 2LL * m->num_sms), 256, 0, s>>>(g);
+  SNO_CUDA(cudaGetLastError());
+  return ETD_OK;
+}
+template <int C, int MP>
+etd_status sno_backward_fused(etd_sno_s* m, const float* u, int B, cudaStream_t s) {
+  const int M = m->M, L = m->L, n = m->n;
+  const long long np = m->npix, M2 = (long long)M * M;
+  const int imgs = B * C;
+  SNO_CUDA(cudaMemsetAsync(m->G, 0, (size_t)m->nparam * sizeof(float), s));
+  // projection: dWq[c] = sum h_L[c] du, dbq = sum du
+  SNO_TRY(chan_reduce(m, m->h[L], m->du, nullptr, B, C, m->oWq, 1, s));
+  SNO_TRY(chan_reduce(m, m->du, nullptr, nullptr, B, 1, m->obq, 1, s));
+  const size_t fsm = ((size_t)MP * ((n + 31) / 32 * 32) + MP * MP) * sizeof(float), psm = 2 * (size_t)M * n * sizeof(float);
+  SNO_CUDA(cudaFuncSetAttribute(grad_field_kernel<MP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm));
+  SNO_CUDA(cudaFuncSetAttribute(modes_pm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+  const int ks = 16;
+  if ((long long)B * ks * C * C > m->part_len) return sfail(ETD_ERR_UNSUPPORTED, "reduction scratch too small");
+  GradPointArgs g{};
+  g.B = B;
+  g.np = np;
+  g.du = m->du;
+  g.Wq = m->W + m->oWq;
+  g.field = m->dh0;
+  for (int l = L - 1; l >= 0; --l) {
+    // dz_l (into z_l) from the layer above
+    g.z = m->z[l];
+    g.out = m->z[l];
+    if (l == L - 1) SNO_TRY((launch_point<C, GRAD_TOP>(m, g, s)));
+    else SNO_TRY((launch_point<C, GRAD_LAYER>(m, g, s)));
+    SNO_TRY(chan_reduce(m, m->z[l], nullptr, nullptr, B, C, m->obp + (long long)l * C, 1, s));
+    grad_weight_kernel<C><<<B * ks, C * C / 8, 0, s>>>(m->z[l], m->h[l], m->part, np, ks);
+    SNO_CUDA(cudaGetLastError());
+    reduce_batch_kernel<<<C * C / 32, 256, 0, s>>>(m->part, m->G + m->oWp + (long long)l * C * C, B * ks, (long long)C * C);
+    SNO_CUDA(cudaGetLastError());
+    // spectral path: dgh = S_M dz S_M^T
+    grad_modes_x_kernel<MP><<<imgs, 128, 0, s>>>(m->z[l], m->S, m->T, n, M);
+    SNO_CUDA(cudaGetLastError());
+    modes_pm_kernel<<<imgs, 64, psm, s>>>(m->S, m->T, m->dgh, n, M, 0);
+    SNO_CUDA(cudaGetLastError());
+    // dWm[l][m][o][c] = sum_b dgh[b][o][m] hh[b][c][m]
+    SNO_TRY(GemmOp(C, C, B, (int)M2)
+                .A(m->dgh, M2, C * M2, 1)
+                .B(m->hh[l], C * M2, M2, 1)
+                .Cm(m->G + m->oWm + (long long)l * M2 * C * C, C, 1, (long long)C * C)
+                .run(s));
+    // dhh[b][c][m] = sum_o bf(Wm[l][m][o][c]) dgh[b][o][m]   (into gh as scratch)
+    {
+      GemmOp o(B, C, C, (int)M2);
+      o.A(m->dgh, C * M2, M2, 1).B(m->W + m->oWm + (long long)l * M2 * C * C, C, 1, (long long)C * C)
+          .Cm(m->gh, C * M2, M2, 1);
+      o.g.round_b = 1;
+      SNO_TRY(o.run(s));
+    }
+    grad_field_kernel<MP><<<imgs, 256, fsm, s>>>(m->gh, m->S, m->dh0, n, M);
+    SNO_CUDA(cudaGetLastError());
+    g.Wp = m->W + m->oWp + (long long)l * C * C;
+    g.dzin = m->z[l];
+  }
+  // lift: dWl[c][0] = sum dh0 u, dWl[c][1] = sum_b a[b] sum_i dh0, dbl[c] = sum dh0 (one set of partial sums for the last two)
+  g.out = m->dh1;
+  SNO_TRY((launch_point<C, GRAD_LIFT>(m, g, s)));
+  SNO_TRY(chan_reduce(m, m->dh1, u, nullptr, B, C, m->oWl, 2, s));
+  SNO_TRY(chan_reduce(m, m->dh1, nullptr, m->a, B, C, m->oWl + 1, 2, s));
+  chan_combine_kernel<<<C, 128, 0, s>>>(m->part, 16, nullptr, B, C, m->G + m->obl, 1);
   SNO_CUDA(cudaGetLastError());
   return ETD_OK;
 }
@@ -444,8 +518,7 @@ etd_status sno_backward(etd_sno_s* m, const float* u, int B, cudaStream_t s) {
       o.g.ksplit = ks;
       o.g.c_ss = (long long)C * C;
       SNO_TRY(o.run(s));
-      reduce_batch_kernel<<<grid_for((long long)C * C), 256, 0, s>>>(m->part, m->G + m->oWp + (long long)l * C * C,
-                                                                    B * ks, (long long)C * C, 0);
+      reduce_batch_kernel<<<(C * C + 31) / 32, 256, 0, s>>>(m->part, m->G + m->oWp + (long long)l * C * C, B * ks, (long long)C * C);
       SNO_CUDA(cudaGetLastError());
     }
     // spectral path: dgh = S_M dz S_M^T
@@ -610,7 +683,12 @@ etd_status etd_sno_train_step(etd_sno m, const float* u, const double* D, const 
   const long long n = (long long)B * m->npix;
   mse_grad_kernel<<<m->lblocks, 256, 0, s>>>(m->uhat, target, m->du, n, m->lpart);
   SNO_CUDA(cudaGetLastError());
-  SNO_TRY(sno_backward(m, u, B, s));
+  if (m->fused_mp && small_modes(m)) {
+    if (m->C == 32) SNO_TRY(m->fused_mp == 16 ? (sno_backward_fused<32, 16>(m, u, B, s)) : (sno_backward_fused<32, 24>(m, u, B, s)));
+    else SNO_TRY(m->fused_mp == 16 ? (sno_backward_fused<16, 16>(m, u, B, s)) : (sno_backward_fused<16, 24>(m, u, B, s)));
+  } else {
+    SNO_TRY(sno_backward(m, u, B, s));
+  }
   if (grads_out) {
     SNO_CUDA(cudaMemcpyAsync(grads_out, m->G, (size_t)m->nparam * sizeof(float), cudaMemcpyDeviceToHost, s));
   } else {

@@ -330,28 +330,47 @@ __global__ void __launch_bounds__(256) chan_dot_kernel(const float* __restrict__
   if (threadIdx.x == 0) part[(long long)bc * gridDim.x + blockIdx.x] = sh[0];
 }
 
-// out[c * stride] (+)= sum_b w[b] sum_k part[(b * C + c) * nblk + k]   (w = NULL: weights 1)
-__global__ void chan_combine_kernel(const float* __restrict__ part, int nblk, const float* __restrict__ w, int B, int C,
-                                    float* __restrict__ out, int stride, int accumulate) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= C) return;
+// out[c * stride] = sum_b w[b] sum_k part[(b * C + c) * nblk + k]   (w = NULL: weights 1), c = blockIdx.x. The inner sums side
+// by side, one field per thread, then the fields in order (as one thread per channel: 28 us at 32 fields, a chain of loads).
+__global__ void __launch_bounds__(128) chan_combine_kernel(const float* __restrict__ part, int nblk, const float* __restrict__ w, int B, int C,
+                                                           float* __restrict__ out, int stride) {
+  __shared__ float ts[128];
+  const int c = blockIdx.x;
   float s = 0.f;
-  for (int b = 0; b < B; ++b) {
+  for (int b0 = 0; b0 < B; b0 += 128) {
+    const int b = b0 + threadIdx.x;
     float t = 0.f;
-    for (int k = 0; k < nblk; ++k) t += part[((long long)b * C + c) * nblk + k];
-    s += (w ? w[b] : 1.f) * t;
+    if (b < B)
+      for (int k = 0; k < nblk; ++k) t += part[((long long)b * C + c) * nblk + k];
+    __syncthreads();
+    ts[threadIdx.x] = t;
+    __syncthreads();
+    if (threadIdx.x == 0)
+      for (int i = 0; i < 128 && b0 + i < B; ++i) s += (w ? w[b0 + i] : 1.f) * ts[i];
   }
-  out[(long long)c * stride] = accumulate ? out[(long long)c * stride] + s : s;
+  if (threadIdx.x == 0) out[(long long)c * stride] = s;
 }
 
-// out[x] = sum_b in[b * X + x] (+ out[x] when accumulate)
-__global__ void reduce_batch_kernel(const float* __restrict__ in, float* __restrict__ out, int B, long long X,
-                                    int accumulate) {
-  for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < X; x += (long long)gridDim.x * blockDim.x) {
-    float s = accumulate ? out[x] : 0.f;
-    for (int b = 0; b < B; ++b) s += in[(long long)b * X + x];
-    out[x] = s;
+// out[x] = sum_b in[b * X + x], in order: 32 columns x per CTA, 64 rows b at a time through shared memory (as one chain of
+// loads per thread: 57 us for 512 rows of 1024)
+__global__ void __launch_bounds__(256) reduce_batch_kernel(const float* __restrict__ in, float* __restrict__ out, int B, long long X) {
+  __shared__ float ts[64][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const long long x = (long long)blockIdx.x * 32 + lane;
+  float s = 0.f;
+  for (int b0 = 0; b0 < B; b0 += 64) {
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int b = b0 + w + 8 * k;
+      ts[w + 8 * k][lane] = b < B && x < X ? in[(long long)b * X + x] : 0.f;
+    }
+    __syncthreads();
+    if (w == 0)
+#pragma unroll 16
+      for (int i = 0; i < 64; ++i) s += ts[i][lane];
   }
+  if (w == 0 && x < X) out[x] = s;
 }
 
 // Adam with bias correction (c1 = 1 - b1^t, c2 = 1 - b2^t)
