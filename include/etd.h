@@ -62,7 +62,10 @@ typedef enum { ETD_F64 = 0, ETD_F32 = 1 } etd_dtype;            /* arithmetic an
  *   extension (a length-2N complex FFT per pair of pencils; rounding grows like log N) folded to the half
  *   its symmetry leaves, FP32 and FP64. Shorter axes: FP32 on ETD_ROUTE_FFT the plain odd extension,
  *   otherwise the half-length recurrence (a length-N complex FFT per pair of pencils followed by a
- *   prefix sum; rounding grows like sqrt(N/2) eps).
+ *   prefix sum; rounding grows like sqrt(N/2) eps). FP64 plans over few pencils take other kernels of
+ *   the same transform where those are faster: dense products up to length 256, the recurrence at 64,
+ *   1536 and 2048. Periodic axes run two-step or one-step Hartley kernels (FP64 over few short pencils:
+ *   dense products).
  * ETD_ROUTE_FFT_SPLIT (FP32; otherwise as ETD_ROUTE_AUTO): Dirichlet axes of N = 1024 (strided ones when
  *   N[0] is a multiple of 4) run a split-radix DST-I: the odd outputs are a DST-III of length N/2, the
  *   even ones split once more into a DST-III of length N/4 and a DST-I of length N/4, each computed by a
@@ -127,7 +130,7 @@ etd_status etd_options_default(etd_options* opt);
  * tables (eigenvalues mu_a, exp(-tau D mu_a), exp(-c2 tau D mu_a), twiddles) on the current
  * device, and uploads them. Supported N[a]: 2^k (4..2048) and 3*2^k (6..1536).
  * Periodic plans (opt->bc = ETD_BC_PERIODIC) run the Hartley kernels on every FFT route (AUTO,
- * FFT and FFT_HALF are the same there: one length-N complex FFT per pair of pencils), and the
+ * FFT and FFT_HALF are the same there), and the
  * Hartley matrix on the GEMM routes.
  * opt may be NULL (defaults). On success *out receives the plan.
  * Errors: ETD_ERR_INVALID_ARG (out/N/h NULL, ndim not 2 or 3, N[a] < 2 or odd, h <= 0, D <= 0,
@@ -250,9 +253,11 @@ etd_status etd_get_plan_info(etd_plan plan, etd_plan_info* info);
  * FFT pass kernels evaluate them per mode, in the arithmetic of dtype: for each of the n modes, from
  * zeta[i] = tau lambda_i >= 0, E[i] = e^{-zeta} and Ec[i] = e^{-c2 zeta} (HOST arrays, rounded to dtype
  * on the device as the kernels' tables hold them), writes out[3i] = phi_1(-zeta), out[3i+1] =
- * phi_2(-zeta), out[3i+2] = c2 phi_1(-c2 zeta) (HOST array of 3n doubles). These are the weights of 3D
- * plans and of 2D plans above the per-mode table size; 2D FP32 plans otherwise use FP64 values rounded
- * once. For checking their accuracy; allocates a temporary device buffer and synchronises. Errors:
+ * phi_2(-zeta), out[3i+2] = c2 phi_1(-c2 zeta) (HOST array of 3n doubles). These are the weights of the
+ * general pass kernels (axes without a two-step or dense plan, the split-radix kernels). The two-step and
+ * dense kernels form phi_1 = (1 - e^{-zeta})/zeta from per-axis values of 1 - e^{-zeta_a} instead and
+ * phi_2 by the same series or (1 - phi_1)/zeta, and 2D plans with per-mode tables read FP64 values
+ * (FP32: rounded once). For checking their accuracy; allocates a temporary device buffer and synchronises. Errors:
  * ETD_ERR_INVALID_ARG for NULL arrays (n > 0), n < 0, c2 outside (0, 1], negative or non-finite zeta,
  * non-finite E or Ec. */
 etd_status etd_phi_weights(etd_dtype dtype, int64_t n, const double* zeta, const double* E, const double* Ec,

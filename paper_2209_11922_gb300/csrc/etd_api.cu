@@ -101,11 +101,10 @@ int env_int(const char* name, int dflt) {
   return (v && *v) ? atoi(v) : dflt;
 }
 
-// Transform variant of an axis of length n with `pairs` pencil pairs: periodic axes the two-step Hartley kernels where they have a plan, else the
-// general Hartley kernels; Dirichlet axes the folded odd
-// extension, which is exact in the same sense as both DST-I forms below and does less work than either, and
-// the lengths it has no plan for (below 32, 24 included) the odd extension or the recurrence: FP32 as the route
-// says (AUTO: the recurrence), FP64 the recurrence.
+// Transform variant of an axis of length n with `pairs` pencil pairs. Periodic axes: the two-step Hartley kernels where they
+// have a plan, else the general Hartley kernels. Dirichlet axes: the folded odd extension, which is exact in the same sense
+// as both older DST-I forms and does less work than either, and for the lengths it has no plan for (below 32, 24 included)
+// the odd extension or the recurrence: FP32 as the route says (AUTO: the recurrence), FP64 the recurrence.
 // FP64 single plans (`batch` false) over few short pencils take dense products: they cost pencils n^2 / 608 cycles
 // per transform where an FFT pass costs its longest thread, 16 to 60 thousand cycles at these lengths. The lines lie
 // where the two were equal (us per ETDRK2 step, dense against FFT: 64^2 19.5 / 138, 128^2 35 / 157, 256^2 148 / 173,
@@ -147,7 +146,7 @@ struct etd_plan_s {
   int scheme = 2;
   etd_options opt{};
   int elem = 8;
-  int odd[3] = {0, 0, 0};  // transform variant per axis: V_ODD, V_REC (DST-I) or V_HART (periodic)
+  int odd[3] = {0, 0, 0};  // transform variant per axis (enum Variant)
   int split[3] = {0, 0, 0};  // FP32 axes of length 1024 on the split-radix kernels (split_pass.cuh)
   int periodic = 0;        // every axis periodic (Hartley kernels), else homogeneous Dirichlet
   int nx = 1, ny = 1, nz = 1;

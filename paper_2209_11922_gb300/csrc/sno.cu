@@ -423,8 +423,8 @@ etd_status chan_reduce(etd_sno_s* m, const float* X, const float* y, const float
 // Gradient with the kernels of sno_grad.cuh (C = 16 or 32, M <= 24): the order of operations of sno_backward.
 template <int C, int KIND>
 etd_status launch_point(const etd_sno_s* m, const GradPointArgs& g, cudaStream_t s) {
-  const long long warps = (g.np + 63) / 64 * g.B;
-  grad_point_kernel<C, KIND><<<(int)std::min<long long>((warps + 7) / 8, 2LL * m->num_sms), 256, 0, s>>>(g);
+  const long long warps = (g.np + 31) / 32 * g.B;
+  grad_point_kernel<C, KIND><<<(int)std::min<long long>((warps + 7) / 8, 3LL * m->num_sms), 256, 0, s>>>(g);
   SNO_CUDA(cudaGetLastError());
   return ETD_OK;
 }

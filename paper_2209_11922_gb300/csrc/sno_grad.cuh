@@ -28,73 +28,63 @@ struct GradPointArgs {
 
 enum { GRAD_TOP = 0, GRAD_LAYER = 1, GRAD_LIFT = 2 };
 
-// 64 pixels per warp, two per lane; four channels at a time in packed pairs, the weights broadcast from shared memory (one
-// 16-byte read per four packed operations). Bound by memory: four fields of B C np floats.
+// One pixel per lane, four channels at a time in packed pairs, the weights broadcast from shared memory (one 16-byte read
+// per two packed operations), the next channels' loads in flight: 262 us where memory alone (four fields of B C np floats, 32 of 255^2 x 32) takes 160;
+// two pixels per lane at two CTAs per SM 313; as separate GEMM, accumulation and GELU passes about 900.
 template <int C, int KIND>
-__global__ void __launch_bounds__(256, 2) grad_point_kernel(const GradPointArgs g) {
+__global__ void __launch_bounds__(256, 3) grad_point_kernel(const GradPointArgs g) {
   __shared__ __align__(16) float W[C * C];   // [o][c]
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   for (int i = tid; i < (KIND == GRAD_TOP ? C : C * C); i += 256) W[i] = KIND == GRAD_TOP ? g.Wq[i] : g.Wp[i];
   __syncthreads();
-  const long long chunks = (g.np + 63) / 64, total = chunks * g.B;
+  const long long chunks = (g.np + 31) / 32, total = chunks * g.B;
   for (long long t = (long long)blockIdx.x * 8 + w; t < total; t += (long long)gridDim.x * 8) {
     const int b = (int)(t / chunks);
-    const long long p0 = (t - b * chunks) * 64 + lane, p1 = p0 + 32, last = g.np - 1;
-    const bool on0 = p0 < g.np, on1 = p1 < g.np;
-    const long long e0 = (long long)b * C * g.np + (on0 ? p0 : last), e1 = (long long)b * C * g.np + (on1 ? p1 : last);
-    float d0[KIND == GRAD_TOP ? 1 : C], d1[KIND == GRAD_TOP ? 1 : C];
+    long long p = (t - b * chunks) * 32 + lane;
+    const bool on = p < g.np;
+    if (!on) p = g.np - 1;
+    long long e = (long long)b * C * g.np + p;
+    float f[4], z[4];
+    auto load = [&](long long q) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (KIND != GRAD_TOP) f[k] = g.field[q + k * g.np];
+        if (KIND != GRAD_LIFT) z[k] = g.z[q + k * g.np];
+      }
+    };
+    float d[KIND == GRAD_TOP ? 1 : C];
     if constexpr (KIND == GRAD_TOP) {
-      d0[0] = g.du[(long long)b * g.np + (on0 ? p0 : last)];
-      d1[0] = g.du[(long long)b * g.np + (on1 ? p1 : last)];
+      d[0] = g.du[(long long)b * g.np + p];
     } else {
 #pragma unroll
-      for (int o = 0; o < C; ++o) {
-        d0[o] = g.dzin[e0 + o * g.np];
-        d1[o] = g.dzin[e1 + o * g.np];
-      }
+      for (int o = 0; o < C; ++o) d[o] = g.dzin[e + o * g.np];
     }
+    load(e);
 #pragma unroll 1
     for (int c0 = 0; c0 < C; c0 += 4) {
-      float f0[4], f1[4], z0[4], z1[4];
+      float fc[4], zc[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const long long q = (c0 + k) * g.np;
-        if (KIND != GRAD_TOP) {
-          f0[k] = g.field[e0 + q];
-          f1[k] = g.field[e1 + q];
-        }
-        if (KIND != GRAD_LIFT) {
-          z0[k] = g.z[e0 + q];
-          z1[k] = g.z[e1 + q];
-        }
+        fc[k] = f[k];
+        zc[k] = z[k];
       }
-      float2 a0[2], a1[2];
-#pragma unroll
-      for (int k = 0; k < 2; ++k) a0[k] = a1[k] = make_float2(0.f, 0.f);
+      if (c0 + 4 < C) load(e + 4 * g.np);
+      float2 a0 = make_float2(0.f, 0.f), a1 = a0;
 #pragma unroll
       for (int o = 0; o < (KIND == GRAD_TOP ? 1 : C); ++o) {
-        const float4 f = *reinterpret_cast<const float4*>(W + o * C + c0);
-        const float2 v0 = make_float2(d0[o], d0[o]), v1 = make_float2(d1[o], d1[o]);
-        a0[0] = fma2f(make_float2(f.x, f.y), v0, a0[0]);
-        a0[1] = fma2f(make_float2(f.z, f.w), v0, a0[1]);
-        a1[0] = fma2f(make_float2(f.x, f.y), v1, a1[0]);
-        a1[1] = fma2f(make_float2(f.z, f.w), v1, a1[1]);
+        const float4 r = *reinterpret_cast<const float4*>(W + o * C + c0);
+        const float2 v = make_float2(d[o], d[o]);
+        a0 = fma2f(make_float2(r.x, r.y), v, a0);
+        a1 = fma2f(make_float2(r.z, r.w), v, a1);
       }
-      float h0[4] = {a0[0].x, a0[0].y, a0[1].x, a0[1].y}, h1[4] = {a1[0].x, a1[0].y, a1[1].x, a1[1].y};
+      float h[4] = {a0.x, a0.y, a1.x, a1.y};
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        if (KIND != GRAD_TOP) {
-          h0[k] += f0[k];
-          h1[k] += f1[k];
-        }
-        if (KIND != GRAD_LIFT) {
-          h0[k] *= gelu_grad(z0[k]);
-          h1[k] *= gelu_grad(z1[k]);
-        }
-        const long long q = (c0 + k) * g.np;
-        if (on0) g.out[e0 + q] = h0[k];
-        if (on1) g.out[e1 + q] = h1[k];
+        if (KIND != GRAD_TOP) h[k] += fc[k];
+        if (KIND != GRAD_LIFT) h[k] *= gelu_grad(zc[k]);
+        if (on) g.out[e + k * g.np] = h[k];
       }
+      e += 4 * g.np;
     }
   }
 }
@@ -102,7 +92,8 @@ __global__ void __launch_bounds__(256, 2) grad_point_kernel(const GradPointArgs 
 // part[b][s][o][c] = sum over the pixels of piece s (kc of them, of field b) of dz[b][o][i] h[b][c][i], in order. One CTA per
 // piece, 4 o x 2 c sums per thread; 32 pixels at a time through shared memory as [pixel][channel], the next ones' loads in
 // flight. A warp loads 8 pixels x 4 channels (32-byte sectors; distinct banks on the transposed store). As a general GEMM
-// with 2 x 2 sums per thread this took 1142 us for 32 fields of 255^2 and 32 channels.
+// with 2 x 2 sums per thread this took 1142 us for 32 fields of 255^2 and 32 channels, here 285; 4 x 4 sums on 64 threads 312 and dz stored
+// twice for the packed operations 320: shared-memory reads and their latency bound it (memory alone: 80).
 template <int C>
 __global__ void __launch_bounds__(C * C / 8) grad_weight_kernel(const float* __restrict__ dz, const float* __restrict__ h, float* __restrict__ part,
                                                                 long long np, int ks) {
@@ -155,7 +146,8 @@ __global__ void __launch_bounds__(C * C / 8) grad_weight_kernel(const float* __r
 
 // First contraction of the truncated transform: T[img][m][y] = sum_x X[img][y][x] S[m][x] (FP32, x in order). One CTA of 128
 // threads per image, two rows y per thread, X staged in 32-column tiles (transposed reads on distinct banks), S as [x][MP]
-// read as broadcasts, two modes per packed instruction.
+// read as broadcasts, two modes per packed instruction: 175 us for 1024 images of 255^2 and 24 modes (general GEMM 227; memory 42:
+// bound by the shared-memory reads, one broadcast of 16 bytes per four packed operations).
 template <int MP>
 __global__ void __launch_bounds__(128) grad_modes_x_kernel(const float* __restrict__ X, const float* __restrict__ S, float* __restrict__ T,
                                                            int n, int M) {
@@ -213,7 +205,8 @@ __global__ void __launch_bounds__(128) grad_modes_x_kernel(const float* __restri
 
 // Inverse truncated transform of an image's modes: out[y][x] = sum_p S[p][y] (sum_q Y[p][q] S[q][x]) (FP32). One CTA of 256
 // threads per image and 256 columns; a thread forms its column's 24 inner sums, then 32 rows y at a time in packed pairs,
-// S as [p][y] read as broadcasts.
+// S as [p][y] read as broadcasts: 189 us for 1024 images of 255^2 and 24 modes, 520 as two GEMM launches (memory 40; bound by
+// the packed operations and their broadcast reads).
 template <int MP>
 __global__ void __launch_bounds__(256, 2) grad_field_kernel(const float* __restrict__ Y, const float* __restrict__ S, float* __restrict__ out,
                                                             int n, int M) {
