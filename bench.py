@@ -43,7 +43,7 @@ def _peaks():
 
 # Sources of the FFT-route pass kernels and of their launch configuration and tables: a change to any
 # of them voids the DRAM-traffic record of profiles/traffic.json.
-PASS_KERNEL_SOURCES = ("dst_engine.cuh", "pass_kernel.cuh", "etd_coeffs.cuh", "etd_api.cu")
+PASS_KERNEL_SOURCES = ("dst_engine.cuh", "fold_dst.cuh", "fold_pass.cuh", "dense_pass.cuh", "pass_kernel.cuh", "etd_coeffs.cuh", "etd_api.cu")
 
 
 def _kernel_source_hash() -> str:

@@ -279,35 +279,33 @@ etd_status make_split_launch(etd_plan_s* pl, int op, int axis, const void* in0, 
   return ETD_OK;
 }
 
-// Dense user field <-> pitched field (PACK / UNPACK): groups of rows of about 1024 elements per block, a thread's
-// elements 256 apart, their loads in flight together.
-constexpr int kPackElems = 1024;
+// Dense user field <-> pitched field (PACK / UNPACK): a row per warp, so that the divisions of the row index are once per
+// row and not once per element, and eight loads per lane in flight.
 template <class T>
 __global__ void __launch_bounds__(256) pack_kernel(const PassArgs<T> A) {
   griddep_wait();
-  constexpr int U = 4;
+  constexpr int U = 8;
   const int cut = A.user_slot;   // 1: Dirichlet (index 0 is the boundary), 0: periodic
-  const int rows = A.ny * A.nz, rpb = A.P, n = rpb * A.nx;   // rows per block
-  const int r0 = blockIdx.x * rpb;
-  for (int i0 = threadIdx.x; i0 < n; i0 += U * 256) {
+  const int r = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (r >= A.ny * A.nz) return;
+  const int z = r / A.ny, y = r - z * A.ny;
+  const bool in = y >= cut && (A.ndim == 2 || z >= cut);   // else a boundary row: zeros, not in the user's field
+  const bool pack = A.op == OP_PACK;
+  const long long user = ((long long)(A.ndim == 3 ? z - cut : 0) * (A.ny - cut) + (y - cut)) * (A.nx - cut) - cut;
+  const T* src = A.in0 + (pack ? user : (long long)r * A.nx);
+  T* dst = A.out0 + (pack ? (long long)r * A.nx : user);
+  if (!pack && !in) return;
+  for (int x0 = threadIdx.x & 31; x0 < A.nx; x0 += 32 * U) {
     T v[U];
-    long long d[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int i = i0 + u * 256, rr = i / A.nx, x = i - rr * A.nx, r = r0 + rr, z = r / A.ny, y = r - z * A.ny;
-      const bool in = i < n && r < rows && x >= cut && y >= cut && (A.ndim == 2 || z >= cut);
-      d[u] = in ? ((long long)(A.ndim == 3 ? z - cut : 0) * (A.ny - cut) + (y - cut)) * (A.nx - cut) + (x - cut) : -1;
-      v[u] = T(0);
-      if (in) v[u] = A.op == OP_PACK ? A.in0[d[u]] : A.in0[(size_t)r0 * A.nx + i];
+      const int x = x0 + 32 * u;
+      v[u] = in && x >= cut && x < A.nx ? src[x] : T(0);
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int i = i0 + u * 256;
-      if (A.op == OP_PACK) {
-        if (i < n && r0 + i / A.nx < rows) A.out0[(size_t)r0 * A.nx + i] = v[u];
-      } else if (d[u] >= 0) {
-        A.out0[d[u]] = v[u];
-      }
+      const int x = x0 + 32 * u;
+      if (x < A.nx && (pack || x >= cut)) dst[x] = v[u];
     }
   }
 }
@@ -446,9 +444,8 @@ etd_status make_launch(etd_plan_s* pl, int op, int axis, const void* in0, const 
     a.in0 = static_cast<const T*>(in0);
     a.out0 = static_cast<T*>(out0);
     a.user_slot = pl->periodic ? 0 : 1;
-    a.P = pl->nx < kPackElems ? kPackElems / pl->nx : 1;
     L.fn = reinterpret_cast<const void*>(&pack_kernel<T>);
-    L.grid = dim3((unsigned)(((long long)pl->ny * pl->nz + a.P - 1) / a.P));
+    L.grid = dim3((unsigned)(((long long)pl->ny * pl->nz + 7) / 8));
     L.block = dim3(256);
     L.smem = 0;
     L.kind = kind;
