@@ -582,7 +582,9 @@ etd_status launch(const Launch& L, cudaStream_t s) {
 // it and its predecessor do not fit on distinct SMs, more of its CTAs fit on an SM than an even spread puts there, and
 // an SM's share loads it: FP64, whose units a warp keeps for 64 cycles, from two warps per SM on, unless
 // equal grids of three or more CTAs per SM follow each other (24 x 256 x 64 ETDRK1
-// 259 us per step with, 149 without; 128 x 192 x 24 599 and 369; 1023^2 298 and 216; many waves lose 0.4%); FP32 CTAs of
+// 259 us per step with, 149 without; 128 x 192 x 24 599 and 369; 1023^2 298 and 216); grids of six or more CTAs per SM spread
+// by themselves (us per run with and without: 64 x 48 x 256 periodic 1787 and 1852, 32 x 48 x 128 periodic 1241 and 1294, against
+// 32 x 128 x 256 periodic 6326 and 6212; a line at four CTAs costs 24 x 256 x 64 1660 -> 2725); FP32 CTAs of
 // 256 threads that would be one per SM, on at least a third of the SMs (1023^2 ETDRK2 31.9 and 28.7).
 void choose_pdl(std::vector<Launch>& step, int num_sms, int elem) {
   for (size_t i = 0; i < step.size(); ++i) {
@@ -594,7 +596,7 @@ void choose_pdl(std::vector<Launch>& step, int num_sms, int elem) {
       cudaGetLastError();
       continue;
     }
-    const bool loads = elem == 8 ? grid * ((threads + 31) / 32) >= 2LL * num_sms && !(grid == prev && grid >= 3LL * num_sms)
+    const bool loads = elem == 8 ? grid < 6LL * num_sms && grid * ((threads + 31) / 32) >= 2LL * num_sms && !(grid == prev && grid >= 3LL * num_sms)
                                  : threads >= 256 && grid <= num_sms && 3 * grid >= num_sms;
     L.pdl = !(grid + prev > num_sms && occ > (grid + num_sms - 1) / num_sms && loads);
   }
