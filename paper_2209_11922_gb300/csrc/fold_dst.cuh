@@ -29,6 +29,8 @@
 // 11 shared-memory accesses and the recurrence 7; here a lone transform makes 2 (A and B sit in registers at
 // both ends where the axis is strided) and the arithmetic is that of a length-N FFT.
 #pragma once
+#include <type_traits>
+
 #include "dst_engine.cuh"
 
 namespace etd {
@@ -89,6 +91,8 @@ constexpr bool fold_has(int n) {
   return n == 32 || n == 48 || n == 64 || n == 96 || n == 128 || n == 192 || n == 256 || n == 384 || n == 512 ||
          n == 768 || n == 1024 || n == 1536 || n == 2048;
 }
+
+constexpr unsigned long long FOLD_MAX_STRIDE = 2048ULL * 2048ULL;   // largest row stride: the z axis behind two axes of 2048
 
 template <class T> __device__ __forceinline__ Cx<T> cmulc(Cx<T> a, Cx<T> b) {   // conj(a) b
   return {a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x};
@@ -272,7 +276,11 @@ template <class T, int N, bool MANY = false> struct Fold {
 
   static __device__ __forceinline__ bool a_on(int jj) { return UA % TPP == 0 || jj < UA; }
   static __device__ __forceinline__ bool b_on(int s) { return SLOTS % TPP == 0 || s < SLOTS; }
-  static __device__ __forceinline__ int partner(int jj) { return jj == 0 ? L / 2 : L - jj; }
+  static constexpr __host__ __device__ __forceinline__ int partner(int jj) { return jj == 0 ? L / 2 : L - jj; }
+  // Rows of step A's inputs: a[r] at jj + r L, b[r] at partner_row(jj) + (PARTNER_STEPS + r) L, where the multiples of L are
+  // the same for every thread.
+  static constexpr int PARTNER_STEPS = 0;
+  static constexpr __host__ __device__ __forceinline__ int partner_row(int jj) { return partner(jj); }
 
   static __device__ __forceinline__ void a(C (&va)[H], C (&vb)[H], int jj, const C* __restrict__ tw) {
     fold_a<T, R, !BIG, UA>(va, vb, jj, tw);
@@ -302,12 +310,12 @@ template <class T, int N, bool MANY = false> struct Fold {
   // Rows (output positions) of the values of B slot s: value i < HV at row1(s) + i STEP, value HV + i at
   // row2(s) + i STEP.
   static constexpr int HV = VB / 2, STEP = BIG ? UT * R : R;
-  static __device__ __forceinline__ int row1(int s) {
+  static constexpr __host__ __device__ __forceinline__ int row1(int s) {
     if constexpr (!BIG) return s;
     const int k = s / UT, t = s % UT;
     return k == 0 ? H * t : R * t + k;
   }
-  static __device__ __forceinline__ int row2(int s) {
+  static constexpr __host__ __device__ __forceinline__ int row2(int s) {
     if constexpr (!BIG) return s == 0 ? H : R - s;
     const int k = s / UT, t = s % UT;
     return k == 0 ? H * (t == 0 ? UT : 2 * UT - t) : R * (UT - 1 - t) + R - k;   // unit 0: the inner transform's rows
@@ -501,10 +509,14 @@ template <class T, int N> struct FoldH {
   static constexpr int LS = L + L / G;
   static_assert(L % G == 0, "slot offsets are compile-time constants");
   static __device__ __forceinline__ bool b_on(int s) { return SLOTS % TPP == 0 || s < SLOTS; }
-  static __device__ __forceinline__ int partner(int jj) { return jj + H * L; }
-  static __device__ __forceinline__ int unit2(int s) { return s == 0 ? H : R - s; }
-  static __device__ __forceinline__ int row1(int s) { return s; }
-  static __device__ __forceinline__ int row2(int s) { return unit2(s); }
+  // b's rows lie N/2 beyond a's: part of the thread's offset (128^3 751 us per 16 steps; as uniform steps 764, 64 x 384 x 384
+  // 570 and 589), but at N = 512, where 32 bits would not hold it behind two axes of 2048, uniform steps.
+  static constexpr bool FAR = (unsigned long long)(H * L + L - 1) * FOLD_MAX_STRIDE * sizeof(T) > 0xffffffffULL;
+  static constexpr int PARTNER_STEPS = FAR ? H : 0;
+  static constexpr __host__ __device__ __forceinline__ int partner_row(int jj) { return FAR ? jj : jj + H * L; }
+  static constexpr __host__ __device__ __forceinline__ int unit2(int s) { return s == 0 ? H : R - s; }
+  static constexpr __host__ __device__ __forceinline__ int row1(int s) { return s; }
+  static constexpr __host__ __device__ __forceinline__ int row2(int s) { return unit2(s); }
   static __device__ __forceinline__ int own_base(int) { return 0; }
   static __device__ __forceinline__ int own_off(int s, int i) { return i < L ? s * LS + i + i / G : unit2(s) * LS + (i - L) + (i - L) / G; }
 
@@ -620,5 +632,34 @@ template <class T, int N> struct FoldH {
     }
   }
 };
+
+// ---------------------------------------------------------------------------------------------
+// Offsets of strided rows. A row's address is a base and a row multiple that are the same for the whole CTA (uniform
+// registers) plus the thread's own part, (row * row stride + column) values with row at most fold_max_row: 32 bits where
+// that fits at the largest row stride, else 64 bits. Only
+// the FP64 plans of N = 1536 and 2048 (rows up to 191 and 255) need 64: 1536 x 1536 x 2048 reaches 4.8e9 bytes, and its six
+// fields (232 GB) fit the card.
+template <class F> __host__ __device__ constexpr int fold_max_row() {
+  int m = 0;
+  for (int s = 0; s < F::SLOTS; ++s) {
+    if (F::row1(s) > m) m = F::row1(s);
+    if (F::row2(s) > m) m = F::row2(s);
+  }
+  for (int jj = 0; jj < F::UA; ++jj) {
+    if (jj > m) m = jj;
+    if (F::partner_row(jj) > m) m = F::partner_row(jj);
+  }
+  return m;
+}
+constexpr int FOLD_MAX_COLUMN = 32;   // columns of a tile: 2 P, P <= 16
+template <class F, class T>
+using FoldOffset =
+    typename std::conditional<((unsigned long long)fold_max_row<F>() * FOLD_MAX_STRIDE + FOLD_MAX_COLUMN) * sizeof(T) <= 0xffffffffULL,
+                              unsigned, unsigned long long>::type;
+template <class F, class T>
+__host__ __device__ __forceinline__ FoldOffset<F, T> fold_offset(int row, size_t stride, int column) {
+  using O = FoldOffset<F, T>;
+  return ((O)row * (O)stride + (O)column) * (O)sizeof(T);
+}
 
 }  // namespace etd

@@ -52,9 +52,8 @@ template <class T> __device__ __forceinline__ void st_pair(T* p, Cx<T> c) {
 }
 
 // Address of a row-segment element: the base and the row step are the same for the whole CTA (uniform registers), the
-// thread's part is a 32-bit byte offset: fewer than L or STEP rows, which is below 2^32 for every plan whose six
-// fields fit the card (the largest, N = 2048 in FP32 with rows 2048^2 elements apart: 255 * 2^24 bytes).
-template <class T> __device__ __forceinline__ T* at_byte(T* base, size_t uniform, unsigned off) {
+// thread's part is fold_offset's.
+template <class T, class O> __device__ __forceinline__ T* at_byte(T* base, size_t uniform, O off) {
   return reinterpret_cast<T*>(const_cast<char*>(reinterpret_cast<const char*>(base)) + uniform + off);
 }
 
@@ -175,6 +174,7 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
       return;
     }
   }
+  [[maybe_unused]] auto row_off = [&](int row) { return fold_offset<F, T>(row, rs, 2 * p); };   // this thread's columns of a row
   // ---- constant tables, before the dependency wait
   {
     const C* gtw = reinterpret_cast<const C*>(A.tw);
@@ -327,13 +327,12 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
   } else {
     // step A's rows, and the stage pass's second operand, in flight together
     const T* src = (OP == OP_S1S || OP == OP_RK1S) ? A.in1 : A.in0;
-    const unsigned oa = ((unsigned)l * (unsigned)rs + 2 * p) * (unsigned)sizeof(T);
-    const unsigned ob = ((unsigned)F::partner(l) * (unsigned)rs + 2 * p) * (unsigned)sizeof(T);
+    const auto oa = row_off(l), ob = row_off(F::partner_row(l));
     const size_t step = (size_t)F::L * rs * sizeof(T);
 #pragma unroll
     for (int r = 0; r < H; ++r) {
       va[r] = ld_pair(at_byte(src + base, r * step, oa));
-      vb[r] = ld_pair(at_byte(src + base, r * step, ob));
+      vb[r] = ld_pair(at_byte(src + base, (F::PARTNER_STEPS + r) * step, ob));
     }
     if constexpr (STAGE && TAB) {
       const T* g = ((OP == OP_S1S || OP == OP_RK1S) ? A.in0 : A.in1) + base;
@@ -343,7 +342,7 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
         if (F::b_on(s)) {
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
-            const unsigned off = ((unsigned)(h ? F::row2(s) : F::row1(s)) * (unsigned)rs + 2 * p) * (unsigned)sizeof(T);
+            const auto off = row_off(h ? F::row2(s) : F::row1(s));
 #pragma unroll
             for (int i = 0; i < HV; ++i)
               cp_async<2 * sizeof(T)>(&own[(q * VB + h * HV + i) * NT + tid], at_byte(g, i * ostep, off));
@@ -383,7 +382,7 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
         F::b_end(bp, s, z, tw);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          const unsigned off = ((unsigned)(h ? F::row2(s) : F::row1(s)) * (unsigned)rs + 2 * p) * (unsigned)sizeof(T);
+          const auto off = row_off(h ? F::row2(s) : F::row1(s));
 #pragma unroll
           for (int i = 0; i < HV; ++i) st_pair(at_byte(g, i * ostep, off), z[h * HV + i]);
         }
@@ -450,7 +449,7 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
     [[maybe_unused]] const T* gu = ((OP == OP_S1S || OP == OP_RK1S) ? A.in0 : A.in1) + base;
     [[maybe_unused]] auto load_u = [&](int s, int c, C (&u)[CH]) {
       const int h = c * CH / HV, i0 = c * CH % HV;
-      const T* g = at_byte(gu, i0 * ostep, ((unsigned)(h ? F::row2(s) : F::row1(s)) * (unsigned)rs + 2 * p) * (unsigned)sizeof(T));
+      const T* g = at_byte(gu, i0 * ostep, row_off(h ? F::row2(s) : F::row1(s)));
 #pragma unroll
       for (int i = 0; i < CH; ++i) u[i] = ld_pair(at_byte(g, i * ostep, 0u));
     };
@@ -489,7 +488,7 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const int row = h ? F::row2(s) : F::row1(s);
-          const unsigned off = ((unsigned)row * (unsigned)rs + 2 * p) * (unsigned)sizeof(T);
+          const auto off = row_off(row);
           const unsigned coff = ((unsigned)row * A.nx + 2 * p) * (unsigned)(FPM * sizeof(T));
           const C* uo = own + (q * VB + h * HV) * NT + tid;
           const unsigned char* wo = reinterpret_cast<const unsigned char*>(wgt) + (size_t)((q * VB + h * HV) * NT + tid) * WB;
@@ -534,7 +533,7 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
           if (c + 1 < NCH) load_u(s, c + 1, un);
           const int h = c * CH / HV, i0 = c * CH % HV;
           const int row = (h ? F::row2(s) : F::row1(s));
-          T* g1 = at_byte(A.out1 + base, i0 * ostep, ((unsigned)row * (unsigned)rs + 2 * p) * (unsigned)sizeof(T));
+          T* g1 = at_byte(A.out1 + base, i0 * ostep, row_off(row));
           C* zo = zs + F::own_off(s, c * CH);
           const int r0 = row + F::STEP * i0;
           const T *tzr = tz + r0, *ter = te + r0, *tcr = tcs + r0, *tmr = tem + r0, *tcmr = tcm + r0;
@@ -590,14 +589,13 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
       stage_out(A.out0);
     } else {
       griddep_launch_dependents();
-      const unsigned oa = ((unsigned)l * (unsigned)rs + 2 * p) * (unsigned)sizeof(T);
-      const unsigned ob = ((unsigned)F::partner(l) * (unsigned)rs + 2 * p) * (unsigned)sizeof(T);
+      const auto oa = row_off(l), ob = row_off(F::partner_row(l));
       const size_t step = (size_t)F::L * rs * sizeof(T);
       T* g = A.out0 + base;
 #pragma unroll
       for (int r = 0; r < H; ++r) {
         st_pair(at_byte(g, r * step, oa), va[r]);
-        st_pair(at_byte(g, r * step, ob), vb[r]);
+        st_pair(at_byte(g, (F::PARTNER_STEPS + r) * step, ob), vb[r]);
       }
     }
   }
