@@ -518,7 +518,7 @@ etd_status make_launch(etd_plan_s* pl, int op, int axis, const void* in0, const 
   }
   a.P = P;
   a.lp = pair_stride(*k, P);
-  L.fn = (op >= 0 && op < OP_COUNT && k->fn_op[op]) ? k->fn_op[op] : k->fn;
+  L.fn = a.coef && k->fn_tab[op] ? k->fn_tab[op] : k->fn;
   L.grid = dim3((unsigned)grid);
   L.block = dim3((unsigned)(P * k->tpp));
   L.smem = pass_smem_bytes(*k, P, two ? 2 : 1);

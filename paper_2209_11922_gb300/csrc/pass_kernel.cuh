@@ -113,13 +113,18 @@ template <> struct V2<double> { using type = double2; };
 // FP32 kernels whose transforms fit are held to 64 registers (two 512-thread CTAs per SM), so that
 // twice as many warps hide shared-memory and FMA latency; the others keep 128.
 template <class T, int N, int VAR> constexpr int pass_min_blocks();
-// Kernels compiled with the table epilogue (per-mode weight tables of 2D plans): the FP64 ones, and the FP32 ones with
-// the full register budget.
-template <class T, int N, int VAR> constexpr bool TABLES_ON() { return sizeof(T) == 8 || pass_min_blocks<T, N, VAR>() == 1; }
+// The table epilogue (template argument TAB: per-mode weight tables of 2D plans). FP32: compiled into the kernels with the
+// full register budget. FP64: into kernels of their own (KernelInfo::fn_tab), which launches with tables take, because in the
+// ones that 3D plans and batches run it costs registers (Hartley N = 64 and 128: 98 and 128 without, 112 and 128 with 60 bytes
+// of spills with it; periodic 24 x 128 x 96 ETDRK1 1404 -> 1354 us per 10 steps, 32 x 128 x 256 ETDRK2 6192 -> 6103); Hartley
+// N = 96 is the exception (96^3 ETDRK2 3470 us per 6 steps with it, 3600 without).
+template <class T, int N, int VAR> constexpr bool TABLES_ON() {
+  return sizeof(T) == 4 ? pass_min_blocks<T, N, VAR>() == 1 : N == 96 && VAR == V_HART;
+}
 // Of those, the FP32 lengths whose tile leaves room for the tile's rows of the tables in shared memory
 // (staged before the dependency wait; the host passes no tables where a launch cannot stage them);
-// longer axes read the tables from global memory.
-template <class T, int N, int VAR> constexpr bool TABLES_STAGED() { return sizeof(T) == 4 && TABLES_ON<T, N, VAR>() && N <= 1536; }
+// longer axes and FP64 read the tables from global memory.
+template <class T, int N, bool TAB> constexpr bool TABLES_STAGED() { return sizeof(T) == 4 && TAB && N <= 1536; }
 // Per-mode weights of one pencil pair at table position m: S1 four values (two per pencil), S2 and RK1
 // two (one per pencil), loaded as 16-byte vectors.
 template <class T> struct PairWeights;
@@ -153,7 +158,7 @@ template <class T> __device__ __forceinline__ void count_step(const PassArgs<T>&
   }
 }
 
-template <class T, int N, int VAR>
+template <class T, int N, int VAR, bool TAB>
 __device__ __forceinline__ void pass_body(const PassArgs<T>& A, const int tile) {
   using L = PairLayout<T, N, VAR>;
   constexpr bool PER = L::HART;   // periodic: no boundary planes, rows or slots
@@ -338,7 +343,7 @@ __device__ __forceinline__ void pass_body(const PassArgs<T>& A, const int tile) 
     const C* gtw = reinterpret_cast<const C*>(A.tw);
     for (int i = tid; i < L::TWN; i += NT) cp_async<2 * sizeof(T)>(&tws[i], &gtw[i]);
   }
-  const bool coef_smem = TABLES_STAGED<T, N, VAR>() && two && A.coef;
+  const bool coef_smem = TABLES_STAGED<T, N, TAB>() && two && A.coef;
   if (two) {
     // the transformed axis's tables, selected without indexing the descriptor's arrays by a run-time
     // value (which would keep a batched kernel's copy of the descriptor in local memory)
@@ -481,8 +486,8 @@ __device__ __forceinline__ void pass_body(const PassArgs<T>& A, const int tile) 
   // values (FP32 plans: rounded once) (A.coef, [y mode][x mode]; e^{-z}, e^{-c2 z} are products of the
   // per-axis factors), with every table load of a chunk of positions issued before the first use. Same
   // effect on the buffers as the epilogue above.
-  // The FP32 kernels with the halved register budget evaluate the weights.
-  constexpr bool TABLES = TABLES_ON<T, N, VAR>();
+  // The kernels without it (TAB) evaluate the weights.
+  constexpr bool TABLES = TAB;
   auto table_epilogue = [&](int kind, C* bpk) {
     if constexpr (TABLES) {
       constexpr int CNT = (N + TPP - 1) / TPP, CH = sizeof(T) == 4 ? 4 : 2;
@@ -492,7 +497,7 @@ __device__ __forceinline__ void pass_body(const PassArgs<T>& A, const int tile) 
       for (int c0 = 0; c0 < CNT; c0 += CH) {
         typename PW::W4 cf4[CH];
         typename PW::W2 cf2[CH];
-        if constexpr (TABLES_STAGED<T, N, VAR>()) {   // staged chunk-major: S1 one pair per chunk, else two
+        if constexpr (TABLES_STAGED<T, N, TAB>()) {   // staged chunk-major: S1 one pair per chunk, else two
 #pragma unroll
           for (int c = 0; c < CH; ++c) {
             const int j = l + (c0 + c) * TPP;
@@ -602,9 +607,9 @@ __device__ __forceinline__ void pass_body(const PassArgs<T>& A, const int tile) 
 }
 
 // One plan: the launch covers the tiles of one field.
-template <class T, int N, int VAR>
+template <class T, int N, int VAR, bool TAB = TABLES_ON<T, N, VAR>()>
 __global__ void __launch_bounds__(512, pass_min_blocks<T, N, VAR>()) pass_kernel(const PassArgs<T> A) {
-  pass_body<T, N, VAR>(A, (int)blockIdx.x);
+  pass_body<T, N, VAR, TAB>(A, (int)blockIdx.x);
 }
 
 // Batches: one launch covers the tiles of many independent problems whose transformed axis has
@@ -619,7 +624,7 @@ __global__ void __launch_bounds__(512, pass_min_blocks<T, N, VAR>())
     if (A.op == OP_ENTRY || A.op == OP_PACK) A.in0 = user[A.user_slot];
     else A.out0 = user[A.user_slot];
   }
-  pass_body<T, N, VAR>(A, m.y);
+  pass_body<T, N, VAR, TABLES_ON<T, N, VAR>()>(A, m.y);
 }
 
 // Host-side description of one instantiation.
@@ -638,8 +643,8 @@ struct KernelInfo {
   int twn;      // twiddle table entries
   int radix[4]; // Stockham radices (0-terminated)
   int min_blocks;  // CTAs per SM the register budget was compiled for
-  // two-step kernels (V_FOLD, V_FOLDH: fn_op and fn_batched_op only)
-  const void* fn_tab[OP_COUNT];  // stage passes reading per-mode weight tables
+  const void* fn_tab[OP_COUNT];  // stage passes reading per-mode weight tables (two-step and FP64 kernels; FP32: fn)
+  // two-step kernels (V_FOLD, V_FOLDM, V_FOLDH: fn_op, fn_batched_op and fn_tab only)
   const void* fn_x;              // OP_TRANSFORM along x
   int max_threads;               // CTA size limit
   int own_vals;                  // values a thread holds after step B
@@ -659,6 +664,9 @@ template <class T, int N, int VAR> KernelInfo kernel_info() {
                N, L::TPP, L::LP, (int)sizeof(T), L::M,
                VAR, L::PADG, L::TWN, {0, 0, 0, 0}, pass_min_blocks<T, N, VAR>()};
   radix_list(k.radix, typename L::Plan::R{});
+  if constexpr (sizeof(T) == 8)
+    for (int op : {OP_RK1, OP_S1, OP_S2, OP_RK1S, OP_S1S, OP_S2S})
+      k.fn_tab[op] = reinterpret_cast<const void*>(&pass_kernel<T, N, VAR, true>);
   return k;
 }
 
