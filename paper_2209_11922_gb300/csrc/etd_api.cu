@@ -94,6 +94,7 @@ struct Launch {
   size_t args_size;
   double alg_bytes;  // algorithmic HBM bytes of this launch (fields read + written)
   bool pdl = true;   // programmatic dependent launch (choose_pdl)
+  enum { GENERAL, TWO_STEP, DENSE } family = GENERAL;
 };
 
 int env_int(const char* name, int dflt) {
@@ -378,6 +379,7 @@ etd_status make_fold_launch(etd_plan_s* pl, const KernelInfo* k, PassArgs<T>& a,
   L.block = dim3((unsigned)(P * k->tpp));
   L.smem = fold_smem_bytes(*k, op, P, a.lp, tab, a.coef_smem != 0);
   L.kind = kind;
+  L.family = Launch::TWO_STEP;
   memcpy(L.args, &a, sizeof(a));
   L.args_size = sizeof(a);
   L.alg_bytes = fields_rw * (double)pl->unknowns * sizeof(T);
@@ -418,6 +420,7 @@ etd_status make_dense_launch(etd_plan_s* pl, PassArgs<double>& a, int kind, doub
   L.block = dim3((unsigned)(W * N * g.KS));
   L.smem = dense_smem_bytes(N, W, g.KS);
   L.kind = kind;
+  L.family = Launch::DENSE;
   memcpy(L.args, &g, sizeof(g));
   L.args_size = sizeof(g);
   L.alg_bytes = fields_rw * (double)pl->unknowns * sizeof(double);
@@ -427,6 +430,7 @@ etd_status make_dense_launch(etd_plan_s* pl, PassArgs<double>& a, int kind, doub
 template <class T>
 etd_status make_launch(etd_plan_s* pl, int op, int axis, const void* in0, const void* in1, void* out0,
                        void* out1, int kind, double fields_rw, Launch& L) {
+  L.family = Launch::GENERAL;
   if constexpr (sizeof(T) == 4) {
     // split-radix kernels, except under a time-dependent source or boundary data (whose passes add
     // to the reaction field with the odd-extension kernels' epilogues)
@@ -576,29 +580,49 @@ etd_status launch(const Launch& L, cudaStream_t s) {
   return ETD_OK;
 }
 
-// Which launches of a time step take programmatic dependent launch. It hides a launch's latency (2 to 4 us of a step),
-// but CTAs that start while their predecessor drains go to the SMs it leaves free, several to one SM, and stay there:
-// where a pass is bound by the warps of the busiest SM it then takes as long as that one. So a launch goes without when
-// it and its predecessor do not fit on distinct SMs, more of its CTAs fit on an SM than an even spread puts there, and
-// an SM's share loads it: FP64, whose units a warp keeps for 64 cycles, from two warps per SM on, unless
-// equal grids of three or more CTAs per SM follow each other (24 x 256 x 64 ETDRK1
-// 259 us per step with, 149 without; 128 x 192 x 24 599 and 369; 1023^2 298 and 216); grids of six or more CTAs per SM spread
-// by themselves (us per run with and without: 64 x 48 x 256 periodic 1787 and 1852, 32 x 48 x 128 periodic 1241 and 1294, against
-// 32 x 128 x 256 periodic 6326 and 6212; a line at four CTAs costs 24 x 256 x 64 1660 -> 2725); FP32 CTAs of
-// 256 threads that would be one per SM, on at least a third of the SMs (1023^2 ETDRK2 31.9 and 28.7).
-void choose_pdl(std::vector<Launch>& step, int num_sms, int elem) {
+// Which launches of a time step take programmatic dependent launch. It hides a launch's latency (2 to 4 us), but CTAs that
+// start while their predecessor drains go to the SMs it leaves free first, several to one SM, and stay there: where a pass is
+// bound by the warps of its busiest SM it then takes as long as that one. That needs a predecessor that does not fill the SMs
+// evenly with the launch's own CTAs beside it, and CTAs of which more fit on an SM than an even spread puts there. What it
+// costs then was measured launch by launch (each on and off, with the step's other launches on and off), for 569 FP64 and
+// 162 FP32 plans:
+//   FP64 FFT passes (a warp holds an FP64 unit for 64 cycles per instruction): up to three times the pass. 512^2 periodic
+//     ETDRK1, 256 one-warp CTAs behind 128: 176 us per step with, 104 without; 128 x 192 x 24, z pass 120 us longer; 1024^2,
+//     x pass 80 us. Behind a grid smaller than the SMs: where the pile puts more warps on a scheduler than the spread.
+//     Behind larger grids: from 4/3 warps per SM on, unless the predecessor's CTAs are far smaller (more than three to one
+//     per SM), up to eight of them per SM on Dirichlet axes and four (and six of its own) on periodic ones.
+//   Not the dense products (short CTAs; 96^2 periodic 29 us per step with, 40 without), and not a general kernel behind an
+//     equal grid of like CTAs, which take the places of those before them (64^3 periodic 27 us per pass with, 30 without).
+//   FP32 passes lose only where CTAs of 256 threads, one to an SM on most SMs, follow about as many (1024^2 ETDRK2 27.5 us
+//     per step without, 28.9 with); smaller grids gain (768^2 ETDRK1 19.4 without, 14.4 with).
+// Summed over those launches, the time lost against the better choice is a fifth of what the attribute everywhere loses in FP64.
+void choose_pdl(std::vector<Launch>& step, int num_sms, int elem, bool periodic) {
+  std::vector<int> occ(step.size(), 0);
+  for (size_t i = 0; i < step.size(); ++i)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[i], step[i].fn, (int)step[i].block.x, step[i].smem) != cudaSuccess) {
+      cudaGetLastError();
+      return;   // every launch keeps the attribute
+    }
+  const long long sms = num_sms;
   for (size_t i = 0; i < step.size(); ++i) {
     Launch& L = step[i];
-    const long long grid = L.grid.x, prev = step[i ? i - 1 : step.size() - 1].grid.x;
-    const int threads = (int)L.block.x;
-    int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, L.fn, threads, L.smem) != cudaSuccess) {
-      cudaGetLastError();
-      continue;
+    const size_t before = i ? i - 1 : step.size() - 1;
+    const long long grid = L.grid.x, prev = step[before].grid.x, warps = grid * ((L.block.x + 31) / 32);
+    const int o = occ[i], op = occ[before];
+    const bool piles = grid + prev > sms && o > (grid + sms - 1) / sms;
+    bool costs;
+    if (elem == 4) {
+      costs = L.block.x >= 256 && grid <= sms && 5 * grid >= 4 * sms && 5 * prev >= 4 * sms && 2 * prev <= 3 * sms;
+    } else if (L.family == Launch::DENSE || (L.family == Launch::GENERAL && grid == prev && (grid < sms ? o < 2 * op && op < 2 * o : 3 * o < 4 * op && 3 * op < 4 * o))) {
+      costs = false;
+    } else if (prev < sms) {   // warps on a scheduler of the busiest SM, piled on the SMs without a predecessor and spread evenly
+      const long long even = (grid + sms - 1) / sms, free = sms - prev, w = (L.block.x + 31) / 32;
+      const long long pile = std::max(even, std::min<long long>(o, (grid + free - 1) / free));
+      costs = (pile * w + 3) / 4 > (even * w + 3) / 4;
+    } else {
+      costs = 3 * o >= op && 3 * warps >= 4 * sms && (periodic ? prev <= 4 * sms && grid < 6 * sms : prev <= 8 * sms);
     }
-    const bool loads = elem == 8 ? grid < 6LL * num_sms && grid * ((threads + 31) / 32) >= 2LL * num_sms && !(grid == prev && grid >= 3LL * num_sms)
-                                 : threads >= 256 && grid <= num_sms && 3 * grid >= num_sms;
-    L.pdl = !(grid + prev > num_sms && occ > (grid + num_sms - 1) / num_sms && loads);
+    L.pdl = !(piles && costs);
   }
 }
 
@@ -750,7 +774,7 @@ etd_status build_step(etd_plan_s* pl) {
   }
 #undef BND
 #undef ADD
-  choose_pdl(pl->step, pl->num_sms, pl->elem);
+  choose_pdl(pl->step, pl->num_sms, pl->elem, pl->periodic != 0);
   return ETD_OK;
 }
 
