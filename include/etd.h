@@ -64,7 +64,7 @@ typedef enum { ETD_F64 = 0, ETD_F32 = 1 } etd_dtype;            /* arithmetic an
  *   otherwise the half-length recurrence (a length-N complex FFT per pair of pencils followed by a
  *   prefix sum; rounding grows like sqrt(N/2) eps). FP64 plans over few pencils take other kernels of
  *   the same transform where those are faster: dense products up to length 256, the recurrence at 64,
- *   1536 and 2048. Periodic axes run two-step or one-step Hartley kernels (FP64 over few short pencils:
+ *   96, 1024, 1536 and 2048. Periodic axes run two-step or one-step Hartley kernels (FP64 over few short pencils:
  *   dense products).
  * ETD_ROUTE_FFT_SPLIT (FP32; otherwise as ETD_ROUTE_AUTO): Dirichlet axes of N = 1024 (strided ones when
  *   N[0] is a multiple of 4) run a split-radix DST-I: the odd outputs are a DST-III of length N/2, the

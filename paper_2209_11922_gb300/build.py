@@ -57,8 +57,7 @@ def generate() -> list:
     for tk, tn in TYPES.items():
         # transform variants (enum Variant of dst_engine.cuh): the two-step kernels (Dirichlet axes 3 and 6, periodic axes 4),
         # and for lengths without a two-step plan 2 Hartley, 1 odd extension (FP32 only; 1024 for the split-radix route's
-        # plans) and 0 half-length recurrence (FP64 64, 1536 and 2048 too, for
-        # few pencils)
+        # plans) and 0 half-length recurrence (FP64 64, 96, 1024, 1536 and 2048 too, for few pencils)
         for v, kind, lengths in (("fold", "V_FOLD", FOLD), ("foldm", "V_FOLDM", FOLDM[tk]), ("foldh", "V_FOLDH", FOLDH[tk])):
             for n in lengths:
                 name = f"kinfo_{tk}_{v}_{n}"
@@ -72,7 +71,7 @@ def generate() -> list:
                 decls.append(f"KernelInfo {name}();")
                 rows.append(f"    {name}(),")
         for v, o in ((("odd", 1), ("rec", 0), ("hart", 2)) if tk == "f32" else (("rec", 0), ("hart", 2))):
-            for n in [m for m in LENGTHS if m not in ([] if v == "hart" else FOLD)] + {"odd": [1024], "rec": [64, 1536, 2048] * (tk == "f64")}.get(v, []):
+            for n in [m for m in LENGTHS if m not in ([] if v == "hart" else FOLD)] + {"odd": [1024], "rec": [64, 96, 1024, 1536, 2048] * (tk == "f64")}.get(v, []):
                 name = f"kinfo_{tk}_{v}_{n}"
                 path = os.path.join(GEN, f"inst_{tk}_{v}_{n}.cu")
                 _write_if_changed(path, (

@@ -109,18 +109,24 @@ int env_int(const char* name, int dflt) {
 // FP64 single plans (`batch` false) over few short pencils take dense products: they cost pencils n^2 / 608 cycles
 // per transform where an FFT pass costs its longest thread, 16 to 60 thousand cycles at these lengths. The lines lie
 // where the two were equal (us per ETDRK2 step, dense against FFT: 64^2 19.5 / 138, 128^2 35 / 157, 256^2 148 / 173,
-// 48^3 108 / 251; 64^3 259 / 232 by the recurrence, 96^3 ETDRK1 490 / 271).
+// 48^3 108 / 251; 64^3 259 / 232 by the recurrence); against the Hartley passes of 32 and 64 they were equal sooner (128 x 32 x
+// 128 periodic ETDRK1 199 / 181 at 2 pairs n^2 = 16.8e6, 32 x 32 x 192 ETDRK2 equal at 6.3e6).
 int dst_variant(const etd_options& o, int axis, int64_t n, int64_t pairs, bool batch) {
   if (o.dtype == ETD_F64 && !batch) {
-    if (n <= 256 && 2 * pairs * n * n <= (n == 64 ? 12000000 : 20000000)) return V_DENSE;
-    // N = 64 up to 4000 pairs, where the folded plan's 4 threads per pair leave schedulers idle, and N = 1536 and 2048
-    // over few pencils: the recurrence's threads hold half the values (8, and 16 against 24 and 32; 64^3 286 us by the
-    // folded plan, 2048 x 64 222 against 307)
-    if (o.bc == ETD_BC_DIRICHLET && ((n == 64 && pairs <= 4000) || ((n == 1536 || n == 2048) && pairs <= 256))) return V_REC;
+    const bool per = o.bc == ETD_BC_PERIODIC;
+    const int64_t line = n == 64 ? (per ? 8000000 : 12000000) : n == 32 && per ? 7000000 : 20000000;
+    if (n <= 256 && 2 * pairs * n * n <= line) return V_DENSE;
+    // The recurrence, whose threads hold half the values, over few pencils: N = 64 up to 4000 pairs (64^3 286 us by the folded
+    // plan, 233), N = 96 on x and z up to 2400 (96 x 24 x 96 ETDRK2 394 us per step by the folded plan, 319; 64 x 64
+    // x 96 440 and 386; on y 192 x 96 x 24 took 7 % more), N = 1024 up to 128 (64 x 1024 244 and 199, 1024 x 128 247 and 210),
+    // N = 1536 and 2048 up to 256 (2048 x 64 307 and 222).
+    if (o.bc == ETD_BC_DIRICHLET && ((n == 64 && pairs <= 4000) || (n == 96 && axis != 1 && pairs <= 2400) ||
+                                        (n == 1024 && pairs <= 128) || ((n == 1536 || n == 2048) && pairs <= 256))) return V_REC;
   }
   // periodic x axes over few pencils whose two-step plan holds 24 or 32 values per thread: the general kernels' 12 to 16
-  // (256 x 24 x 64 255 us per 12 steps against 217, 384 x 192 125 against 111; N = 128 holds 16 and is faster)
-  if (o.bc == ETD_BC_PERIODIC && axis == 0 && !batch && (n == 96 || n >= 192) && pairs < 1100) return V_HART;
+  // (256 x 24 x 64 255 us per 12 steps against 217, 384 x 192 125 against 111, 96 x 32 x 96 15.8 us per step against 14.5 at
+  // 1536 pairs, equal at 3072; N = 128 holds 16 and is faster)
+  if (o.bc == ETD_BC_PERIODIC && axis == 0 && !batch && (n == 96 || n >= 192) && pairs < 2000) return V_HART;
   if (o.bc == ETD_BC_PERIODIC) return foldh_has(o.dtype == ETD_F32 ? 4 : 8, (int)n, pairs) ? V_FOLDH : V_HART;
   // few pencils: the plans with many threads (256^2 876 -> 636 us per 40 steps, 768 x 192 560 -> 476; N = 128 gains nothing)
   if (o.dtype == ETD_F32 && !batch && foldm_has((int)n) && pairs <= 2000) return V_FOLDM;
