@@ -46,11 +46,6 @@ __device__ __forceinline__ void mma16816_init(float (&d)[4], const uint32_t (&a)
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(c0), "f"(c1));
 }
 
-// gelu(z) = z/2 (1 + erf(z/sqrt2)) = max(z, 0) - (|z|/2) erfc(|z|/sqrt2) with
-// erfc(t/sqrt2) = 2^{-q(t)}, q(t)/t a degree-9 polynomial fitted on [0, 6.5] (minimax in the error of the result; beyond,
-// q keeps growing and the term vanishes). Over N(0, 2^2) and [-9, 9] its error against 64 bits is 4.1e-8 rms, 2.4e-7
-// at most; z/2 (1 + erff(z/sqrt2)) in FP32 gives 5.4e-8 and 4.5e-7.
-// (Scalar instructions: packed ones cost more register moves around the MMA fragments than they saved.)
 union F2 {
   float2 f;
   unsigned long long u;
@@ -63,15 +58,16 @@ __device__ __forceinline__ float2 fma2f(float2 a, float2 b, float2 c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.u) : "l"(x.u), "l"(y.u), "l"(z.u));
   return r.f;
 }
-__device__ __forceinline__ float2 mul2f(float2 a, float2 b) {
-  F2 x, y, r;
-  x.f = a;
-  y.f = b;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.u) : "l"(x.u), "l"(y.u));
-  return r.f;
-}
-__device__ __forceinline__ float gelu_erfc(float z) {
-  const float t = fabsf(z);
+// gelu(z) = z/2 (1 + erf(z/sqrt2)) = max(z, 0) - (|z|/2) erfc(|z|/sqrt2) with
+// erfc(t/sqrt2) = 2^{-q(t)}, q(t)/t a degree-9 polynomial fitted on [0, 6.5] (minimax in the error of the result; beyond,
+// q keeps growing and the term vanishes). Over N(0, 2^2) and [-9, 9] its error against 64 bits is 3.6e-8 and 4.9e-8 rms,
+// 2.4e-7 at most; z/2 (1 + erff(z/sqrt2)) in FP32 gives 5.1e-8, 6.7e-8 and 4.9e-7.
+// (Scalar instructions: packed ones cost more register moves around the MMA fragments than they saved.)
+// SAFE: gelu(+inf) = +inf, as in the training forward; without, NaN (the vanishing term is inf * 0). The last layer, whose
+// values the projection adds up, takes it; in the others, whose infinities the next transform turns into NaN all over the field
+// either way, the one instruction more was 1.8 % of a forward pass (1356 -> 1380 us at 64 fields of 255^2 and 32 channels).
+template <bool SAFE> __device__ __forceinline__ float gelu_erfc(float z) {
+  const float t = fabsf(SAFE ? fminf(z, 3.4028235e38f) : z);
   float p = 2.7615620012966247e-08f;
   p = fmaf(p, t, -8.48519789542479e-07f);
   p = fmaf(p, t, 1.105071078200126e-05f);
@@ -87,9 +83,9 @@ __device__ __forceinline__ float gelu_erfc(float z) {
   asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(r) : "f"(z));
   return fmaf(-0.5f * t, e, r);
 }
-__device__ __forceinline__ void gelu4(float2 (&z)[4]) {
+template <bool SAFE> __device__ __forceinline__ void gelu4(float2 (&z)[4]) {
 #pragma unroll
-  for (int k = 0; k < 4; ++k) z[k] = make_float2(gelu_erfc(z[k].x), gelu_erfc(z[k].y));
+  for (int k = 0; k < 4; ++k) z[k] = make_float2(gelu_erfc<SAFE>(z[k].x), gelu_erfc<SAFE>(z[k].y));
 }
 
 struct LayerArgs {
@@ -372,7 +368,7 @@ __global__ void __launch_bounds__(256, 2) layer_kernel(const LayerArgs g) {
       for (int i = 0; i < NJ / 2; ++i) {
         float2 z[4] = {make_float2(acc[2 * i][0], acc[2 * i][1]), make_float2(acc[2 * i + 1][0], acc[2 * i + 1][1]),
                        make_float2(acc[2 * i][2], acc[2 * i][3]), make_float2(acc[2 * i + 1][2], acc[2 * i + 1][3])};
-        gelu4(z);
+        gelu4<LAST>(z);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           sa = fmaf(wq[2 * i + h][1], z[h].y, fmaf(wq[2 * i + h][0], z[h].x, sa));
@@ -395,7 +391,7 @@ __global__ void __launch_bounds__(256, 2) layer_kernel(const LayerArgs g) {
       for (int i = 0; i < NJ / 2; ++i) {
         float2 z[4] = {make_float2(acc[2 * i][0], acc[2 * i][1]), make_float2(acc[2 * i + 1][0], acc[2 * i + 1][1]),
                        make_float2(acc[2 * i][2], acc[2 * i][3]), make_float2(acc[2 * i + 1][2], acc[2 * i + 1][3])};
-        gelu4(z);
+        gelu4<LAST>(z);
         if (va) *reinterpret_cast<float4*>(oa + odd * LX * C + 16 * i) = make_float4(z[0].x, z[0].y, z[1].x, z[1].y);
         if (vb) *reinterpret_cast<float4*>(ob + odd * LX * C + 16 * i) = make_float4(z[2].x, z[2].y, z[3].x, z[3].y);
         *reinterpret_cast<uint2*>(ta + 32 * i) = va ? make_uint2(bf2(z[0].x, z[0].y), bf2(z[1].x, z[1].y)) : make_uint2(0u, 0u);
