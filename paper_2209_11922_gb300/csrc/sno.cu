@@ -364,6 +364,11 @@ etd_status launch_layer(const LayerArgs& g, cudaStream_t s) {
   SNO_CUDA(cudaGetLastError());
   return ETD_OK;
 }
+// Shared memory of kernels whose need depends on n (at most 255 here) stays within the 48 KB that a launch may ask for without
+// the attribute: a limit set to one operator's size would refuse a larger operator's launch in another thread.
+constexpr size_t kPlainSmem = 48 * 1024;
+template <int MP> constexpr size_t grad_field_smem(int n) { return ((size_t)MP * ((n + 31) / 32 * 32) + MP * MP) * sizeof(float); }
+static_assert(modes_y_smem(255, 24) <= kPlainSmem && grad_field_smem<24>(255) <= kPlainSmem, "no attribute needed");
 template <int C, int MP>
 etd_status sno_infer(etd_sno_s* m, const float* u, int B, float* out, cudaStream_t s) {
   const int n = m->n, M = m->M, L = m->L;
@@ -384,7 +389,6 @@ etd_status sno_infer(etd_sno_s* m, const float* u, int B, float* out, cudaStream
   g.out = out;
   lift_modes_kernel<C, MP><<<dim3(std::min((n + 7) / 8, std::max(1, 4 * m->num_sms / B)), B), 256, 0, s>>>(g);
   SNO_CUDA(cudaGetLastError());
-  SNO_CUDA(cudaFuncSetAttribute(modes_y_kernel<MP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)modes_y_smem(n, MP)));
   for (int l = 0; l < L; ++l) {
     modes_y_kernel<MP><<<dim3((C * MP + 127) / 128, B), 256, modes_y_smem(n, MP), s>>>(m->S, m->Ty, m->hh[0], B, n, M, C);
     SNO_CUDA(cudaGetLastError());
@@ -437,8 +441,7 @@ etd_status sno_backward_fused(etd_sno_s* m, const float* u, int B, cudaStream_t 
   // projection: dWq[c] = sum h_L[c] du, dbq = sum du
   SNO_TRY(chan_reduce(m, m->h[L], m->du, nullptr, B, C, m->oWq, 1, s));
   SNO_TRY(chan_reduce(m, m->du, nullptr, nullptr, B, 1, m->obq, 1, s));
-  const size_t fsm = ((size_t)MP * ((n + 31) / 32 * 32) + MP * MP) * sizeof(float), psm = 2 * (size_t)M * n * sizeof(float);
-  SNO_CUDA(cudaFuncSetAttribute(grad_field_kernel<MP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm));
+  const size_t fsm = grad_field_smem<MP>(n), psm = 2 * (size_t)M * n * sizeof(float);
   SNO_CUDA(cudaFuncSetAttribute(modes_pm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   const int ks = 16;
   if ((long long)B * ks * C * C > m->part_len) return sfail(ETD_ERR_UNSUPPORTED, "reduction scratch too small");

@@ -492,7 +492,7 @@ __global__ void __launch_bounds__(256) modes_y_kernel(const float* __restrict__ 
     if (2 * i + 1 < M) hh[((size_t)((2 * i + 1) * M + q) * B + b) * C + c] = bf16_round(acc[i].y + o.y);
   }
 }
-inline size_t modes_y_smem(int n, int MP) { return (size_t)(n * MP > 128 * MP ? n * MP : 128 * MP) * sizeof(float); }
+constexpr size_t modes_y_smem(int n, int MP) { return (size_t)(n * MP > 128 * MP ? n * MP : 128 * MP) * sizeof(float); }
 
 // Per-mode channel mix: gh[mode][b][o] = sum_c bf(Wm[mode][o][c]) hh[mode][b][c] (FP32, channels in order). One CTA per
 // mode, o = tid % C.

@@ -1,4 +1,6 @@
-"""The operator's inference at the edges of its arithmetic."""
+"""The operator at the edges of its arithmetic, and two operators in two threads."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -36,3 +38,39 @@ def test_activation_of_an_overflowed_value(C, M, value):
     loss, _ = s.gradient(u, D, u)
     assert loss == np.inf or loss >= float(value) ** 2 * 0.99
     s.close()
+
+
+def test_operators_of_two_sizes_in_two_threads():
+    """Two operators whose launches need different amounts of shared memory, used from two threads on two streams: every call
+    succeeds and gives the result it gives alone (no call sets a kernel's limit to its own size, which a launch of the other
+    operator would then exceed)."""
+    ops = [_op(32, 16, 24, 1, 1), _op(256, 16, 24, 12, 1)]
+    want = []
+    for s, u, D in ops:
+        want.append((s.forward(u, D).clone(), s.gradient(u, D, 0.5 * u)[1]["Wm"].copy()))
+    torch.cuda.synchronize()
+    errors = []
+    go = threading.Barrier(2)
+
+    def work(k):
+        s, u, D = ops[k]
+        stream = torch.cuda.Stream()
+        try:
+            go.wait()
+            with torch.cuda.stream(stream):
+                tgt = 0.5 * u
+                for _ in range(1500 if k == 0 else 150):
+                    out = s.forward(u, D, stream=stream)
+                    _, g = s.gradient(u, D, tgt, stream=stream)
+                stream.synchronize()
+            assert torch.equal(out, want[k][0]) and np.array_equal(g["Wm"], want[k][1])
+        except BaseException as e:   # noqa: BLE001 - reported by the main thread
+            errors.append((k, repr(e)))
+    ts = [threading.Thread(target=work, args=(k,)) for k in range(2)]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    assert not errors, errors
+    for s, _, _ in ops:
+        s.close()
