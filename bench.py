@@ -467,6 +467,19 @@ def run_batched(args, bw):
     return 0
 
 
+def _sno_forward_bytes(B: int, n: int, C: int, M: int, L: int) -> float:
+    """Algorithmic bytes of one inference forward of B fields n x n (FP32 activations). Spectral part of a layer, either form:
+    mesh contraction of the truncated transform (T out), its second contraction (T in, modes out), mode mix (modes in and
+    out), first inverse contraction (modes in, T out), T in again. Fused layers (C = 16 or 32, M <= 24, n <= 256,
+    sno_layer.cuh): h once out and once in between two layers; u into the lift's transform, the first layer and the residual,
+    u_hat out. Otherwise h_0 out, h in twice, z out and in, h' out per layer, h_L in."""
+    npix = n * n
+    spectral = L * (4 * C * M * n + 4 * C * M * M)
+    if C in (16, 32) and M <= 24 and n <= 256:
+        return 4.0 * B * (4 * npix + 2 * (L - 1) * C * npix + spectral)
+    return 4.0 * B * (npix + C * npix + 5 * L * C * npix + spectral + C * npix + 2 * npix)
+
+
 def measure_sno(args, sw) -> dict:
     """Parareal with the trained SNO as coarse propagator against the plain batched ETDRK2 solver on
     B problems at N x N (windows x window steps). Training (data from the plain solver, Adam) runs
@@ -544,13 +557,7 @@ def measure_sno(args, sw) -> dict:
     g = torch.empty_like(u0)
     ms_coarse = timed(lambda: sno.forward(u0, D, out=g, stream=stream), args.steps)
     fl = 2.0 * B * sw.C * sw.L * (2 * (n * n * sw.M + n * sw.M * sw.M) + sw.C * n * n)   # GEMM flops
-    # Algorithmic bytes of one inference forward (FP32 activations): lift (u in, h_0 out); per layer the
-    # mesh contraction of the truncated transform (h in, T out), its second contraction (T in, modes
-    # out), the mode mix (modes in and out), the first inverse contraction (modes in, T out), the second
-    # (T in, z out) and the pointwise mix with GELU (h and z in, h' out); projection (h_L, u in, u_hat
-    # out).
-    npix, C, M, L = n * n, sw.C, sw.M, sw.L
-    fwd_bytes = 4.0 * B * (npix + C * npix + L * (5 * C * npix + 4 * C * M * n + 4 * C * M * M) + C * npix + 2 * npix)
+    fwd_bytes = _sno_forward_bytes(B, n, sw.C, sw.M, sw.L)
     hbm_peak, hbm_src = _peaks()
     achieved = fwd_bytes / (ms_coarse * 1e-3) / 1e9
     line = {
