@@ -69,7 +69,7 @@ struct etd_sno_s {
   float* T = nullptr;      // transform scratch [Bmax][C][n][M] (also [M][n])
   float* gh = nullptr;     // [Bmax][C][M][M]
   float* dgh = nullptr;
-  float* dh0 = nullptr;    // gradient ping-pong [Bmax][C][npix]
+  float* dh0 = nullptr;    // gradient ping-pong [Bmax][C][npix]; inference: the layers' contractions along x (Ty, Tx)
   float* dh1 = nullptr;
   float* uhat = nullptr;   // [Bmax][npix] (training)
   float* du = nullptr;     // [Bmax][npix]
@@ -82,8 +82,6 @@ struct etd_sno_s {
   bool tc = false;
   int fused_mp = 0;        // inference by the fused layers (sno_layer.cuh): modes per axis padded to 16 or 24, 0: not
   uint2* Sf = nullptr;     // S_M as bf16 fragments
-  float* Ty = nullptr;     // [Bmax][n y][C][MP]
-  float* Tx = nullptr;     // [Bmax][n x][C][MP]
   int num_sms = 148;
   int* err = nullptr;      // set by a tensor-core kernel whose wait ran out
 };
@@ -271,7 +269,7 @@ etd_status upload_feature(etd_sno_s* m, const double* D, int B, cudaStream_t s) 
 namespace {
 
 void sno_free(etd_sno_s* m) {
-  float* bufs[] = {m->W, m->G, m->Mo, m->Ve, m->S, m->a, m->T, m->Ty, m->Tx, m->gh, m->dgh, m->dh0, m->dh1, m->uhat, m->du, m->part};
+  float* bufs[] = {m->W, m->G, m->Mo, m->Ve, m->S, m->a, m->T, m->gh, m->dgh, m->dh0, m->dh1, m->uhat, m->du, m->part};
   for (float* p : bufs)
     if (p) cudaFree(p);
   for (float* p : m->h) cudaFree(p);
@@ -372,6 +370,7 @@ static_assert(modes_y_smem(255, 24) <= kPlainSmem && grad_field_smem<24>(255) <=
 template <int C, int MP>
 etd_status sno_infer(etd_sno_s* m, const float* u, int B, float* out, cudaStream_t s) {
   const int n = m->n, M = m->M, L = m->L;
+  float *Ty = m->dh0, *Tx = m->dh1;   // [B][n y][C][MP], [B][n x][C][MP]
   LayerArgs g{};
   g.B = B;
   g.n = n;
@@ -382,19 +381,19 @@ etd_status sno_infer(etd_sno_s* m, const float* u, int B, float* out, cudaStream
   g.bl = m->W + m->obl;
   g.S = m->S;
   g.Sf = m->Sf;
-  g.T = m->Ty;
-  g.Tf = m->Tx;
+  g.T = Ty;
+  g.Tf = Tx;
   g.Wq = m->W + m->oWq;
   g.bq = m->W + m->obq;
   g.out = out;
   lift_modes_kernel<C, MP><<<dim3(std::min((n + 7) / 8, std::max(1, 4 * m->num_sms / B)), B), 256, 0, s>>>(g);
   SNO_CUDA(cudaGetLastError());
   for (int l = 0; l < L; ++l) {
-    modes_y_kernel<MP><<<dim3((C * MP + 127) / 128, B), 256, modes_y_smem(n, MP), s>>>(m->S, m->Ty, m->hh[0], B, n, M, C);
+    modes_y_kernel<MP><<<dim3((C * MP + 127) / 128, B), 256, modes_y_smem(n, MP), s>>>(m->S, Ty, m->hh[0], B, n, M, C);
     SNO_CUDA(cudaGetLastError());
     mode_mix_kernel<C><<<M * M, 256, 0, s>>>(m->W + m->oWm + (long long)l * M * M * C * C, m->hh[0], m->gh, B);
     SNO_CUDA(cudaGetLastError());
-    modes_x_kernel<MP><<<dim3((C * MP + 255) / 256, B, (n + 63) / 64), 256, 0, s>>>(m->S, m->gh, m->Tx, B, n, M, C);
+    modes_x_kernel<MP><<<dim3((C * MP + 255) / 256, B, (n + 63) / 64), 256, 0, s>>>(m->S, m->gh, Tx, B, n, M, C);
     SNO_CUDA(cudaGetLastError());
     g.Wp = m->W + m->oWp + (long long)l * C * C;
     g.bp = m->W + m->obp + (long long)l * C;
@@ -590,6 +589,13 @@ etd_status etd_sno_create(etd_sno* out, int N, int C, int M, int L, int max_batc
     return st;
   };
   const long long act = (long long)max_batch * C * m->npix;
+  // Fused inference layers: channel counts and mode counts whose fragments fit the registers (C = 16 or 32, M <= 24)
+  // and rows whose bf16 S_M fits beside the tiles; they round the operands that the tensor-core path rounds, so only
+  // where that path runs.
+  m->tc = m->n <= 256 && C <= 256 && M <= 256;
+  if (m->tc && (C == 16 || C == 32) && M <= 24) m->fused_mp = M <= 16 ? 16 : 24;
+  // the contractions of the fused layers are wider than a field only where n < fused_mp
+  const long long act_t = std::max(act, (long long)max_batch * m->n * C * m->fused_mp);
   etd_status st;
   if ((st = sno_alloc(&m->W, m->nparam)) != ETD_OK || (st = sno_alloc(&m->G, m->nparam)) != ETD_OK ||
       (st = sno_alloc(&m->Mo, m->nparam)) != ETD_OK || (st = sno_alloc(&m->Ve, m->nparam)) != ETD_OK ||
@@ -597,7 +603,7 @@ etd_status etd_sno_create(etd_sno* out, int N, int C, int M, int L, int max_batc
       (st = sno_alloc(&m->T, (long long)max_batch * C * m->n * M)) != ETD_OK ||
       (st = sno_alloc(&m->gh, (long long)max_batch * C * M2)) != ETD_OK ||
       (st = sno_alloc(&m->dgh, (long long)max_batch * C * M2)) != ETD_OK ||
-      (st = sno_alloc(&m->dh0, act)) != ETD_OK || (st = sno_alloc(&m->dh1, act)) != ETD_OK ||
+      (st = sno_alloc(&m->dh0, act_t)) != ETD_OK || (st = sno_alloc(&m->dh1, act_t)) != ETD_OK ||
       (st = sno_alloc(&m->uhat, (long long)max_batch * m->npix)) != ETD_OK ||
       (st = sno_alloc(&m->du, (long long)max_batch * m->npix)) != ETD_OK)
     return bail(st);
@@ -625,18 +631,11 @@ etd_status etd_sno_create(etd_sno* out, int N, int C, int M, int L, int max_batc
           (float)(std::sqrt(2.0 / N) * std::sin(M_PI * (double)(((long long)(p + 1) * (j + 1)) % (2LL * N)) / N));
   if (cudaMemcpy(m->S, hs.data(), hs.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess)
     return bail(sfail(ETD_ERR_CUDA, "upload of the mode matrix"));
-  m->tc = m->n <= 256 && C <= 256 && M <= 256;
-  // Fused inference layers: channel counts and mode counts whose fragments fit the registers (C = 16 or 32, M <= 24)
-  // and rows whose bf16 S_M fits beside the tiles; they round the operands that the tensor-core path rounds, so only
-  // where that path runs.
-  if (m->tc && (C == 16 || C == 32) && M <= 24) {
-    m->fused_mp = M <= 16 ? 16 : 24;
-    const long long cnt = (long long)max_batch * m->n * C * m->fused_mp;
+  if (m->fused_mp) {
     const std::vector<uint2> f = s_fragments(hs, M, m->fused_mp, m->n);
     if (cudaMalloc(&m->Sf, f.size() * sizeof(uint2)) != cudaSuccess ||
         cudaMemcpy(m->Sf, f.data(), f.size() * sizeof(uint2), cudaMemcpyHostToDevice) != cudaSuccess)
       return bail(sfail(ETD_ERR_OOM, "mode-matrix fragments"));
-    if ((st = sno_alloc(&m->Ty, cnt)) != ETD_OK || (st = sno_alloc(&m->Tx, cnt)) != ETD_OK) return bail(st);
   }
   int dev = 0;
   cudaGetDevice(&dev);
