@@ -82,6 +82,21 @@ template <class T> __device__ __forceinline__ Cx<T> phi2_series2(Cx<T> z) {
 // phi_2 = (1 - phi_1)/zeta, below zeta = 1 its series, evaluated only in warps holding such a mode. What bounds the
 // stage passes of 3D plans and batches is this evaluation's instruction count: against phi_1 and phi_1(c2) by
 // series and an IEEE reciprocal per mode it is a third.
+// 1 - e^{-(zeta + zeta')} of two modes from p = 1 - e^{-zeta} and m = 1 - e^{-zeta'}.
+template <class T> __device__ __forceinline__ Cx<T> join_m(T m, Cx<T> p) { return fma2(Cx<T>{-m, -m}, p, p + Cx<T>{m, m}); }
+// phi_1 -> 1 as zeta -> 0 (periodic mode 0; the Dirichlet boundary slot, whose values are zero); the bounds keep the
+// reciprocal finite.
+template <class T> constexpr T zeta_lo() { return sizeof(T) == 4 ? T(1e-30) : T(1e-290); }
+template <class T> __device__ __forceinline__ Cx<T> bounded_zeta(Cx<T> zt) {
+  constexpr T lo = zeta_lo<T>(), hi = T(1) / lo;
+  return Cx<T>{fmin(fmax(zt.x, lo), hi), fmin(fmax(zt.y, lo), hi)};
+}
+// m / zeta, rz = 1 / bounded_zeta(zt); at0: the value at zeta = 0.
+template <class T> __device__ __forceinline__ Cx<T> phi1_pair(Cx<T> zt, Cx<T> rz, Cx<T> m, T at0) {
+  constexpr T lo = zeta_lo<T>();
+  const Cx<T> q = mul2(m, rz);
+  return Cx<T>{zt.x > lo ? q.x : at0, zt.y > lo ? q.y : at0};
+}
 template <class T> __device__ __forceinline__ Cx<T> phi2_pair(Cx<T> zeta, Cx<T> rz, Cx<T> p1, unsigned act) {
   const Cx<T> one{T(1), T(1)};
   Cx<T> p2 = mul2(one - p1, rz);
@@ -437,8 +452,8 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
         if constexpr (!TAB) {
           const T z = A.zeta[1][o], m = A.em[1][o], cm = A.cm[1][o];
           pz = pz + C{z, z};
-          pm = fma2(C{-m, -m}, pm, pm + C{m, m});
-          pcm = fma2(C{-cm, -cm}, pcm, pcm + C{cm, cm});
+          pm = join_m(m, pm);
+          pcm = join_m(cm, pcm);
         }
       }
     }
@@ -541,20 +556,15 @@ __device__ __forceinline__ void fold_body(const PassArgs<T>& A, const int tile, 
           for (int i = 0; i < CH; ++i) {
             const C u = uc[i], w = zo[i];
             const T zj = tzr[F::STEP * i], mj = tmr[F::STEP * i];
-            // phi_1 -> 1 as zeta -> 0 (periodic mode 0; the Dirichlet boundary slot, whose values are zero); the bounds
-            // keep the reciprocal finite
-            constexpr T lo = sizeof(T) == 4 ? T(1e-30) : T(1e-290), hi = T(1) / lo;
-            const C zt = pz + C{zj, zj}, zeta{fmin(fmax(zt.x, lo), hi), fmin(fmax(zt.y, lo), hi)};
-            const C rz = rcp2(zeta), q1 = mul2(fma2(C{-mj, -mj}, pm, pm + C{mj, mj}), rz);
-            const C p1{zt.x > lo ? q1.x : T(1), zt.y > lo ? q1.y : T(1)};
+            const C zt = pz + C{zj, zj}, zeta = bounded_zeta(zt), rz = rcp2(zeta);
+            const C p1 = phi1_pair(zt, rz, join_m(mj, pm), T(1));
             const unsigned act = __activemask();
             C o0, o1;
             if constexpr (OP == OP_S1S) {
               const T ej = ter[F::STEP * i], cj = tcr[F::STEP * i], cmj = tcmr[F::STEP * i];
               const C p2 = phi2_pair<T>(zeta, rz, p1, act);
               // c2 phi_1(-c2 zeta) = (1 - e^{-c2 zeta}) / zeta
-              const C q2 = mul2(fma2(C{-cmj, -cmj}, pcm, pcm + C{cmj, cmj}), rz);
-              const C t1{zt.x > lo ? q2.x : A.c2, zt.y > lo ? q2.y : A.c2};
+              const C t1 = phi1_pair(zt, rz, join_m(cmj, pcm), A.c2);
               o0 = fma2(mul2(C{tau, tau}, t1), w, mul2(mul2(pc, C{cj, cj}), u));
               o1 = fma2(mul2(C{tau, tau}, fma2(C{-inv_c2, -inv_c2}, p2, p1)), w, mul2(mul2(pe, C{ej, ej}), u));
             } else if constexpr (OP == OP_RK1S) {
