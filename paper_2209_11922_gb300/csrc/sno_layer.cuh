@@ -14,7 +14,7 @@
 // by whole accumulators in tensor memory would need both products materialised; at 2-10 flops per byte the tensor
 // rate does not matter. h' goes through a bf16 tile in shared memory to the next layer's first contraction
 //   T[y][c][m] = sum_x bf(h'[y][x][c]) bf(S[m][x])                              A: the tile transposed, B: S
-// whose accumulators a warp keeps for its 4 rows y over the whole loop along x. The operands rounded to bf16, and the
+// whose accumulators a warp keeps for its 2 rows y over the whole loop along x. The operands rounded to bf16, and the
 // FP32 ones, are those of the unfused kernels.
 #pragma once
 #include <cuda_bf16.h>
@@ -197,10 +197,11 @@ __global__ void __launch_bounds__(256) lift_modes_kernel(const LayerArgs g) {
   }
 }
 
-// One layer: CTA = 32 rows y of one field, 16 warps, steps of 8 columns x; warp w handles column w / 2 of the step for
-// the 16-row tile w % 2, and after every second step rows 2w, 2w + 1 of the contraction along x. The tiles of
-// h (from HBM) arrive by cp.async two steps ahead, those of Tf (from L2) one: a step is about a thousand cycles, less than
-// the latency of its loads, and with both one step ahead a layer took 310 us.
+// One layer: CTA = 16 rows y of one field, 8 warps, steps of 8 columns x; warp w handles column w of the step for all
+// 16 rows, and after every second step rows 2w, 2w + 1 of the contraction along x. The tiles of h (from HBM) and Tf (from
+// L2) arrive by cp.async one step ahead in two stages; what hides the rest of their latency is the second CTA of the SM.
+// 251 us for an inner layer of 64 fields of 255^2 and 32 channels (0.67 of the copy bandwidth), 256 for the first, which
+// reads only u: the instruction stream (GELU, conversions, fragment moves) bounds both.
 template <int C, int MP, bool FIRST, bool LAST>
 __global__ void __launch_bounds__(256, 2) layer_kernel(const LayerArgs g) {
   constexpr int NJ = C / 8, KC = C / 16, KS = (MP + 15) / 16, MJ = MP / 8, NT = 256;
