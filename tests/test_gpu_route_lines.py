@@ -51,3 +51,17 @@ def test_fp32_dirichlet(N):
 @pytest.mark.parametrize("N", F32_PERIODIC, ids=lambda n: "x".join(map(str, n)))
 def test_fp32_periodic(N):
     _check(N, "periodic", "f32")
+
+
+@pytest.mark.parametrize("N", [(64, 64), (1024, 1024), (96, 48), (32, 48, 64)], ids=lambda n: "x".join(map(str, n)))
+def test_fft_routes_are_one_route_from_length_32(N):
+    """ETD_ROUTE_FFT and ETD_ROUTE_FFT_HALF run AUTO's kernels on axes of 32 and more: the same bits, hence AUTO's 1e-5."""
+    from paper_2209_11922_gb300.etd import Plan
+    U = inputs.uniform_field(inputs.field_shape(N, "dirichlet"), -0.9, 0.9, 77).astype(np.float32)
+    got = []
+    for route in ("auto", "fft", "fft_half"):
+        with Plan(N, 1e-3, 1e-2, scheme=2, dtype="f32", route=route) as pl:
+            d = torch.from_numpy(np.ascontiguousarray(U)).cuda()
+            pl.run(d, 5)
+            got.append(d)
+    assert torch.equal(got[0], got[1]) and torch.equal(got[0], got[2])
